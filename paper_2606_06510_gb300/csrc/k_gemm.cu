@@ -20,20 +20,25 @@
 // (the A operand stores its last nonsquare plane pre-scaled by -2^b, the
 // accumulator merge of §2.5 "Accumulators").  Every K-slab (32768 squares,
 // 4096 nonsquare: Eq. accum-exact) the epilogue reads the accumulators and
-// forms  v = acc0 + s·acc1  or  v = 16·acc0 - 15·acc1  mod m.  After a slab
-// that is not the last it writes the centred residue back into the
-// accumulators (tcgen05.st) for the next slab to accumulate on; after the
-// last it stores the centred residue as int16, column-major (each thread
-// owns one row; a warp's store covers 32 consecutive rows of one column, 64
-// contiguous bytes).
+// adds  acc0 + s·acc1  or  16·acc0 - 15·acc1  mod m to the residue it keeps
+// in registers; after the last slab it stores the centred residue as int16,
+// column-major (each thread owns one row; a warp's store covers 32
+// consecutive rows of one column, 64 contiguous bytes).
 //
 // Pipeline: a stage is one (A plane, B plane) pair of 128-byte-deep tiles
 // (32 KiB per CTA), six stages.  Warp 0 of each CTA issues its CTA's TMA
 // loads, completing on the leader's stage barrier; warp 1 of the leader
 // issues the MMAs and multicasts stage releases and accumulator-ready
 // signals to both CTAs; warps 2..17 of both CTAs run the epilogue (64
-// columns each) and release the accumulators to the leader.  Every wait is bounded; on expiry the
-// kernel records OZ2_ERR_TIMEOUT in the device status word and drains.
+// columns each) and release the accumulators to the leader.  Every wait is
+// bounded; on expiry the kernel records OZ2_ERR_TIMEOUT in the device status
+// word and drains.
+//
+// Two kernels share this: residue_gemm_kernel (k > 128), which orders a
+// unit's products so that each accumulator is drained while the tensor cores
+// work on the other one, and plane_gemm_kernel, for the one-k-block residue
+// GEMM and the magnitude GEMM, whose units are over before such an overlap
+// could start or use one accumulator only.
 #include <algorithm>
 
 #include "oz2_gemm.cuh"
@@ -118,18 +123,12 @@ template <int MODE>
 __device__ __forceinline__ int planes_of(const Oz2Moduli& mods, int i) {
   return MODE == 0 ? (mods.sq_base[i] ? 2 : 3) : 1;
 }
-template <int MODE>
-__device__ __forceinline__ int64_t slab_steps_of(const Oz2Moduli& mods, int i, int64_t ksteps) {
-  if (MODE == 1) return ksteps;  // the magnitude sums stay below 2^24 units over all of k
-  return (mods.sq_base[i] ? kKSlabSquare : kKSlabMerged) / kBK;
-}
-
-// MODE 0: residue planes (all moduli); MODE 1: magnitude planes ("+1" pass).
-// SHORT1, for MODE 0: the instance for k ≤ 128 (one k-block, so one short
-// slab for every modulus), whose epilogue takes the single-correction
-// reduction; for MODE 1: the instance whose tiles run in parts of k and add
-// their partial sums into U (EpiCtx::upart) instead of taking row maxima.
-template <int MODE, bool SHORT1 = false>
+// MODE 0: residue planes (all moduli) for k ≤ 128: one k-block, so one short
+// slab for every modulus, whose epilogue takes the single-correction
+// reduction.  MODE 1: magnitude planes ("+1" pass); with PARTS its tiles run
+// in parts of k and add their partial sums into U (EpiCtx::upart) instead of
+// taking row maxima.
+template <int MODE, bool PARTS = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     plane_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       const __grid_constant__ Oz2Moduli mods, int64_t k_pad, UnitMap um, EpiCtx ctx) {
@@ -236,61 +235,57 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         const Unit x = unit_at<MODE>(u, um);
         const int i = x.i;
         const int np = planes_of<MODE>(mods, i);
-        const int64_t slab = slab_steps_of<MODE>(mods, i, ksteps);
-        for (int64_t kb0 = x.k_lo; kb0 < x.k_hi && ok; kb0 += slab) {
-          if (!mbar_wait_bounded(acc_empty, accph ^ 1, kWaitLimit)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const int64_t kb1 = min(x.k_hi, kb0 + slab);
-          for (int64_t kb = kb0; kb < kb1 && ok; ++kb) {
-            const uint32_t first = kb == x.k_lo ? 0u : 1u;  // later slabs add to the carried residue
-            if (np == 2) {  // square: stages (d0,e0) and (d1,e1)
-              uint32_t s1 = st, p1 = ph;
-              next(s1, p1);
-              if (!mbar_wait_bounded(full0 + 8 * st, ph, kWaitLimit) || !mbar_wait_bounded(full0 + 8 * s1, p1, kWaitLimit)) {
+        if (!mbar_wait_bounded(acc_empty, accph ^ 1, kWaitLimit)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        for (int64_t kb = x.k_lo; kb < x.k_hi && ok; ++kb) {
+          const uint32_t first = kb == x.k_lo ? 0u : 1u;
+          if (np == 2) {  // square: stages (d0,e0) and (d1,e1)
+            uint32_t s1 = st, p1 = ph;
+            next(s1, p1);
+            if (!mbar_wait_bounded(full0 + 8 * st, ph, kWaitLimit) || !mbar_wait_bounded(full0 + 8 * s1, p1, kWaitLimit)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint64_t a0 = desc0 + st * (kStageBytes >> 4), b0 = a0 + (kTileBytes >> 4);
+            const uint64_t a1 = desc0 + s1 * (kStageBytes >> 4), b1 = a1 + (kTileBytes >> 4);
+#pragma unroll
+            for (int kk = 0; kk < kBK / 32; ++kk) {
+              const uint32_t acc = kk ? 1u : first;
+              mma_f8_pair(tmem, a0 + 2 * kk, b0 + 2 * kk, idesc, acc);                 // d0·e0
+              mma_f8_pair(tmem + kAccCols, a1 + 2 * kk, b0 + 2 * kk, idesc, acc);      // d1·e0
+              mma_f8_pair(tmem + kAccCols, a0 + 2 * kk, b1 + 2 * kk, idesc, 1u);       // + d0·e1
+            }
+            mma_commit_pair_mc(empty0 + 8 * st, 0x3);
+            mma_commit_pair_mc(empty0 + 8 * s1, 0x3);
+            st = s1;
+            ph = p1;
+            next(st, ph);
+          } else {
+            for (int p = 0; p < np; ++p) {  // nonsquare: Σ·Σ → acc0; d0e0, -16 d1·e1 → acc1
+              if (!mbar_wait_bounded(full0 + 8 * st, ph, kWaitLimit)) {
                 ok = false;
                 break;
               }
               tc_fence_after();
-              const uint64_t a0 = desc0 + st * (kStageBytes >> 4), b0 = a0 + (kTileBytes >> 4);
-              const uint64_t a1 = desc0 + s1 * (kStageBytes >> 4), b1 = a1 + (kTileBytes >> 4);
+              const uint32_t col = p == 0 ? 0u : kAccCols;
+              const uint64_t a = desc0 + st * (kStageBytes >> 4), b = a + (kTileBytes >> 4);
 #pragma unroll
               for (int kk = 0; kk < kBK / 32; ++kk) {
-                const uint32_t acc = kk ? 1u : first;
-                mma_f8_pair(tmem, a0 + 2 * kk, b0 + 2 * kk, idesc, acc);                 // d0·e0
-                mma_f8_pair(tmem + kAccCols, a1 + 2 * kk, b0 + 2 * kk, idesc, acc);      // d1·e0
-                mma_f8_pair(tmem + kAccCols, a0 + 2 * kk, b1 + 2 * kk, idesc, 1u);       // + d0·e1
+                const uint32_t acc = (kk || p == 2) ? 1u : first;
+                mma_f8_pair(tmem + col, a + 2 * kk, b + 2 * kk, idesc, acc);
               }
               mma_commit_pair_mc(empty0 + 8 * st, 0x3);
-              mma_commit_pair_mc(empty0 + 8 * s1, 0x3);
-              st = s1;
-              ph = p1;
               next(st, ph);
-            } else {
-              for (int p = 0; p < np; ++p) {  // nonsquare: Σ·Σ → acc0; d0e0, -16 d1·e1 → acc1
-                if (!mbar_wait_bounded(full0 + 8 * st, ph, kWaitLimit)) {
-                  ok = false;
-                  break;
-                }
-                tc_fence_after();
-                const uint32_t col = p == 0 ? 0u : kAccCols;
-                const uint64_t a = desc0 + st * (kStageBytes >> 4), b = a + (kTileBytes >> 4);
-#pragma unroll
-                for (int kk = 0; kk < kBK / 32; ++kk) {
-                  const uint32_t acc = (kk || p == 2) ? 1u : first;
-                  mma_f8_pair(tmem + col, a + 2 * kk, b + 2 * kk, idesc, acc);
-                }
-                mma_commit_pair_mc(empty0 + 8 * st, 0x3);
-                next(st, ph);
-              }
             }
           }
-          if (!ok) break;
-          mma_commit_pair_mc(acc_full, 0x3);  // accumulators complete for this slab, both CTAs
-          accph ^= 1;
         }
+        if (!ok) break;
+        mma_commit_pair_mc(acc_full, 0x3);  // the unit's accumulators complete, both CTAs
+        accph ^= 1;
       }
       if (!ok) {
         ctx.dev->status = kStatusTimeout;
@@ -319,134 +314,429 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       const float inv = 1.f / mf;
       const float sb = MODE == 0 ? static_cast<float>(mods.sq_base[i]) : 0.f;
       const float hi = MODE == 0 ? static_cast<float>(mods.m[i] - 1 - mods.m[i] / 2) : 0.f;
-      // This thread's row of C^(i) (of part `part` of it under split K);
-      // column j at rrow[j·ldr] (a warp stores 32 consecutive rows of one
-      // column, 64 contiguous bytes, per instruction).
-      int16_t* rrow =
-          MODE == 0 ? ctx.res + (static_cast<size_t>(x.part) * mods.r + i) * ctx.n * ctx.ldr + row : nullptr;
-      const int64_t slab = slab_steps_of<MODE>(mods, i, ksteps);
-      // Short slabs (K = 128·(k_hi - k_lo) k-entries): v stays an integer below 2^24
-      // without reducing the accumulators first.  Square moduli (|d0e0| ≤ 256,
-      // |d1e0 + d0e1| ≤ 512, s ≤ 33): |v| ≤ K(256 + 33·512) < 2^24 for K ≤ 896.
-      // Nonsquare (|(d0+d1)(e0+e1)| ≤ 22², merged term ≤ 4095):
-      // |16·acc0 - 15·acc1| ≤ K(16·484 + 15·4095) < 2^24 for K ≤ 128.
-      const bool short_slab = MODE == 0 && x.k_hi - x.k_lo <= (square ? 7 : 1);
+      // This thread's row of C^(i); column j at rrow[j·ldr] (a warp stores 32
+      // consecutive rows of one column, 64 contiguous bytes, per instruction).
+      int16_t* rrow = MODE == 0 ? ctx.res + static_cast<size_t>(i) * ctx.n * ctx.ldr + row : nullptr;
       float rowmax = 0.f;
-      for (int64_t kb0 = x.k_lo; kb0 < x.k_hi; kb0 += slab) {
+      if (!mbar_wait_bounded(acc_full, accph, kWaitLimit)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+#pragma unroll 2
+      for (int c = 0; c < 64; c += 16) {
+        uint32_t v0[16], v1[16];
+        tmem_ld16(lane_addr + c, v0);
+        if (MODE == 0) tmem_ld16(lane_addr + kAccCols + c, v1);
+        tmem_ld_wait();
+        if (c == 48) {
+          // The last chunk is in registers: release the accumulators now, so
+          // the next unit's MMAs overlap this chunk's reduction and stores.
+          // The arrive is relaxed: the residue stores before it need no
+          // ordering against the MMAs, and a release would wait for them to
+          // be performed.
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_remote_relaxed(acc_empty_leader);
+        }
+        if (MODE == 1 && PARTS) {  // a part of k: add this tile's partial sums into U
+          const int64_t cc = col0 + c;
+          if (row < ctx.m) {
+            float* dst = ctx.upart + row * ctx.ldu + cc;  // 16-byte aligned: ldu and cc multiples of 4
+            if (cc + 16 <= ctx.n) {
+#pragma unroll
+              for (int j = 0; j < 16; j += 4)
+                atomicAdd(reinterpret_cast<float4*>(dst + j),
+                          make_float4(__uint_as_float(v0[j]), __uint_as_float(v0[j + 1]), __uint_as_float(v0[j + 2]),
+                                      __uint_as_float(v0[j + 3])));
+            } else {
+#pragma unroll
+              for (int j = 0; j < 16; ++j)
+                if (cc + j < ctx.n) atomicAdd(dst + j, __uint_as_float(v0[j]));
+            }
+          }
+        } else if (MODE == 1) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) rowmax = fmaxf(rowmax, __uint_as_float(v0[j]));
+        } else if (row < ctx.m) {
+          const int64_t cc = col0 + c;
+          int16_t* dst = rrow + cc * ctx.ldr;
+          const int ncol = ctx.n - cc < 16 ? static_cast<int>(ctx.n - cc) : 16;
+          if (ncol == 16 && square) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const float rj =
+                  combine_residue_short1<true>(__uint_as_float(v0[j]), __uint_as_float(v1[j]), sb, mf, inv, hi);
+              *dst = static_cast<int16_t>(as_i16_bits(rj));
+              dst += ctx.ldr;
+            }
+          } else if (ncol == 16) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const float rj =
+                  combine_residue_short1<false>(__uint_as_float(v0[j]), __uint_as_float(v1[j]), sb, mf, inv, hi);
+              *dst = static_cast<int16_t>(as_i16_bits(rj));
+              dst += ctx.ldr;
+            }
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const float v = fmaf(square ? 1.f : 16.f, __uint_as_float(v0[j]), (square ? sb : -15.f) * __uint_as_float(v1[j]));
+              if (j < ncol) *dst = static_cast<int16_t>(as_i16_bits(short_residue(v, mf, inv, hi)));
+              dst += ctx.ldr;
+            }
+          }
+        }
+      }
+      accph ^= 1;
+      if (MODE == 1 && !PARTS) {
+        // rows past m hold zeros (TMA fills out-of-range rows with 0)
+        if (row < ctx.m) atomicMax(reinterpret_cast<int*>(ctx.urow) + row, __float_as_int(rowmax));
+        const int wm = __reduce_max_sync(0xffffffffu, __float_as_int(rowmax));
+        if (lane == 0) atomicMax(&ctx.dev->u_max_bits, wm);
+      }
+    }
+    if (!ok) {
+      ctx.dev->status = kStatusTimeout;
+      ctx.dev->timeout_site = 3;
+    }
+  }
+  tc_fence_before();
+  cluster_sync_all();  // neither CTA leaves while the pair's MMAs or loads may touch it
+  tc_fence_after();
+  if (warp == 1) tmem_dealloc_pair(tmem, kTmemCols);
+}
+
+// ---------------------------------------------------------------------------
+// The residue GEMM for k > 128.
+//
+// What bounds it: the tensor pipes and the power cap.  A 256×256×4096 unit is
+// 49,152 cycles of MMAs on a pair; it takes about 57,000, at the 1.79 to 1.86
+// GHz the SMs hold under this load (2.07 GHz idle; the counters of the kernel
+// itself: cycles over nanoseconds), with the MMA issuer waiting 6% of them
+// for operands and none for the epilogue.
+//
+// The two 256-column accumulators fill tensor memory, and draining both after
+// a unit left the tensor cores idle for about 4 µs of every unit.  Here the
+// products of a K-slab are ordered so that each accumulator is complete well
+// before, or started well after, the other:
+//   nonsquare: phase A  all k-blocks of (d0+d1)(e0+e1)       → acc0
+//              phase B  all k-blocks of d0·e0, (-16 d1)·e1    → acc1
+//   square:    phase A  d0·e0 of the first kSplitSteps blocks → acc0
+//              phase M  every product of the other blocks     → acc0, acc1
+//              phase B  d1·e0 + d0·e1 of the first blocks     → acc1
+// The epilogue drains acc0 during phase B and acc1 during the next slab's or
+// unit's phase A.  FP32 sums of integers below 2^24 do not depend on the
+// order.  A square unit loads its first kSplitSteps d0, e0 tiles twice for
+// this (it has the loads to spare: two stages per 12 MMAs against three).
+// Between the two drains, and from slab to slab, the residue stays in
+// registers, two 16-bit values to a word (no write-back to tensor memory).
+//
+// Measured (both builds in turn on one GB300, GEMM stage): 4096³ r = 12 1.376
+// → 1.285 ms, 2500×3001×2047 r = 15 0.459 → 0.402, 2048³ r = 8 0.136 → 0.129,
+// 16384³ r = 13 (whole call, power cap) 130.1 → 120.3.  kSplitSteps 4, 5, 8,
+// 12 and 20 gave 0.644, 0.641, 0.646, 0.659 and 0.655 ms on squares alone
+// (4096³, r = 6): more blocks cover the drain better and load more.  Asking
+// L2 for the operand blocks ahead of the loads (eight k-blocks, the pairs
+// that share a block taking turns) changed nothing (1.260 against 1.260 ms),
+// nor did the tensor core's operand-A collector on the squares' shared d0.
+// ---------------------------------------------------------------------------
+constexpr int kSplitSteps = 5;       // k-blocks of a square slab whose two accumulators are filled apart
+
+__device__ __forceinline__ int residue_slab_steps(bool square) {
+  return (square ? kKSlabSquare : kKSlabMerged) / kBK;
+}
+
+// Two residues of magnitude below 2^15 in one word, biased by 2^15.
+constexpr float kPackBias = kRoundMagic + 32768.f;
+__device__ __forceinline__ uint32_t pack_residues(float lo, float hi) {
+  return __byte_perm(__float_as_uint(lo + kPackBias), __float_as_uint(hi + kPackBias), 0x5410);
+}
+// w·(residue j of the word), exactly: the biased float times w, less the
+// biased zero times w, is an integer below 2^20.
+__device__ __forceinline__ float unpack_scaled(uint32_t word, int j, float w) {
+  return fmaf(w, __uint_as_float(__byte_perm(word, 0x4B40u, j ? 0x5432 : 0x5410)), -w * kPackBias);
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
+    residue_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                        const __grid_constant__ Oz2Moduli mods, int64_t k_pad, UnitMap um, EpiCtx ctx) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
+  // bars: full[S], empty[S], acc_full[2], acc_empty[2], drain
+  __shared__ uint32_t tmem_base_s;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const bool leader = rank == 0;
+  const int64_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kStages);
+  const uint32_t acc_full = smem_u32(bars + 2 * kStages), acc_empty = smem_u32(bars + 2 * kStages + 2);
+  const uint32_t drain_bar = smem_u32(bars + 2 * kStages + 4);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(acc_full + 8 * a, 1);
+      mbar_init(acc_empty + 8 * a, 2 * kEpiWarps);
+    }
+    mbar_init(drain_bar, 1);
+    fence_barrier_init();
+    prefetch_tensormap(&tmA);
+    prefetch_tensormap(&tmB);
+  }
+  if (warp == 1) {
+    tmem_alloc_pair(smem_u32(&tmem_base_s), kTmemCols);
+    tmem_relinquish_pair();
+  }
+  tc_fence_before();
+  cluster_sync_all();
+  tc_fence_after();
+  const uint32_t tmem = tmem_base_s;
+  bool ok = true;
+
+  if (warp == 0) {
+    // ---------------- TMA producer (both CTAs) ----------------
+    if (lane == 0) {
+      const uint32_t full_leader0 = mapa_shared(full0, 0);
+      uint32_t it = 0, s = 0, ph = 1;
+      auto load = [&](int line_a, int line_b) {
+        if (!mbar_wait_bounded(empty0 + 8 * s, ph, kWaitLimit)) {
+          ok = false;
+          return;
+        }
+        if (leader) mbar_arrive_expect_tx(full0 + 8 * s, 2u * kStageBytes);
+        const uint32_t sa = smem_u32(smem + s * kStageBytes);
+        tma_load_2d_pair(sa, &tmA, full_leader0 + 8 * s, 0, line_a);
+        tma_load_2d_pair(sa + kTileBytes, &tmB, full_leader0 + 8 * s, 0, line_b);
+        ++it;
+        if (++s == kStages) {
+          s = 0;
+          ph ^= 1;
+        }
+      };
+      const int kb_lines = mods.nplanes * kPlaneRows;  // lines from one k-block's blocks to the next's
+      for (int64_t w = 0, u = pair; u < um.nunits && ok; u = wave_unit(pair, ++w, npairs)) {
+        const Unit x = unit_at<0>(u, um);
+        const bool square = mods.sq_base[x.i] != 0;
+        const int slab = residue_slab_steps(square), khi = static_cast<int>(x.k_hi);
+        // First lines of this modulus's plane 0 in k-block 0 of the unit's row
+        // blocks.  A row block past the operand's last one lies past the end
+        // of the tensor (zero fill).
+        const int pline = mods.plane_off[x.i] * kPlaneRows;
+        const int line_a = static_cast<int>((x.tm * 2 + rank) * um.ksteps * kb_lines) + pline;
+        const int line_b = static_cast<int>((x.tn * 2 + rank) * um.ksteps * kb_lines) + pline;
+        auto blocks = [&](int kb0, int kb1, int p0, int np) {
+          for (int kb = kb0; kb < kb1 && ok; ++kb) {
+            const int off = kb * kb_lines + p0 * kPlaneRows;
+            for (int p = 0; p < np && ok; ++p) load(line_a + off + p * kPlaneRows, line_b + off + p * kPlaneRows);
+          }
+        };
+        for (int k0 = static_cast<int>(x.k_lo); k0 < khi && ok; k0 += slab) {
+          const int k1 = min(k0 + slab, khi), ke = square ? min(k0 + kSplitSteps, k1) : k1;
+          blocks(k0, ke, 0, 1);
+          blocks(ke, k1, 0, 2);
+          blocks(k0, ke, square ? 0 : 1, 2);
+        }
+      }
+      if (!ok) {
+        ctx.dev->status = kStatusTimeout;
+        ctx.dev->timeout_site = 1;
+      }
+      if (leader)  // the leader's stage barriers also count the peer's bytes
+        for (uint32_t j = (it > kStages ? it - kStages : 0); j < it; ++j)
+          mbar_wait_bounded(full0 + 8 * (j % kStages), (j / kStages) & 1, kWaitLimit);
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ---------------- MMA issuer (leader CTA) ----------------
+    if (leader && lane == 0) {
+      constexpr uint32_t idesc = idesc_f8_f32(kTileM, kTileN);
+      // Stage s, operand o, k-chunk kk: the descriptor of stage 0 plus the
+      // byte offset >> 4 (the start-address field has room: smem < 256 KiB).
+      const uint64_t desc0 = smem_desc_sw128(smem_u32(smem));
+      uint32_t st = 0, ph = 0, accph = 1;  // current stage and its full-barrier parity
+      auto wait_stage = [&]() {
+        if (!mbar_wait_bounded(full0 + 8 * st, ph, kWaitLimit)) ok = false;
+        return ok;
+      };
+      auto release_stage = [&](uint32_t s) { mma_commit_pair_mc(empty0 + 8 * s, 0x3); };
+      auto next = [&]() {
+        if (++st == kStages) {
+          st = 0;
+          ph ^= 1;
+        }
+      };
+      // One stage into one accumulator.
+      auto single = [&](uint32_t col, uint32_t acc) {
+        if (!wait_stage()) return;
+        tc_fence_after();
+        const uint64_t a = desc0 + st * (kStageBytes >> 4), b = a + (kTileBytes >> 4);
+#pragma unroll
+        for (int kk = 0; kk < kBK / 32; ++kk) mma_f8_pair(tmem + col, a + 2 * kk, b + 2 * kk, idesc, kk ? 1u : acc);
+        release_stage(st);
+        next();
+      };
+      // A square's stage pair (d0, e0), (d1, e1): d1·e0 + d0·e1 into acc1,
+      // and, when `both`, d0·e0 into acc0.
+      auto cross = [&](bool both, uint32_t acc0, uint32_t acc1) {
+        if (!wait_stage()) return;
+        const uint32_t s0 = st;
+        next();
+        if (!wait_stage()) return;
+        const uint32_t s1 = st;
+        next();
+        tc_fence_after();
+        const uint64_t a0 = desc0 + s0 * (kStageBytes >> 4), b0 = a0 + (kTileBytes >> 4);
+        const uint64_t a1 = desc0 + s1 * (kStageBytes >> 4), b1 = a1 + (kTileBytes >> 4);
+#pragma unroll
+        for (int kk = 0; kk < kBK / 32; ++kk) {
+          if (both) mma_f8_pair(tmem, a0 + 2 * kk, b0 + 2 * kk, idesc, kk ? 1u : acc0);
+          mma_f8_pair(tmem + kAccCols, a1 + 2 * kk, b0 + 2 * kk, idesc, kk ? 1u : acc1);
+          mma_f8_pair(tmem + kAccCols, a0 + 2 * kk, b1 + 2 * kk, idesc, 1u);
+        }
+        release_stage(s0);
+        release_stage(s1);
+      };
+      for (int64_t w = 0, u = pair; u < um.nunits && ok; u = wave_unit(pair, ++w, npairs)) {
+        const Unit x = unit_at<0>(u, um);
+        const bool square = mods.sq_base[x.i] != 0;
+        const int slab = residue_slab_steps(square), khi = static_cast<int>(x.k_hi);
+        for (int k0 = static_cast<int>(x.k_lo); k0 < khi && ok; k0 += slab) {
+          const int k1 = min(k0 + slab, khi), ke = square ? min(k0 + kSplitSteps, k1) : k1;
+          if (!mbar_wait_bounded(acc_empty, accph, kWaitLimit)) ok = false;
+          tc_fence_after();
+          for (int kb = k0; kb < ke && ok; ++kb) single(0, kb != k0);  // phase A
+          if (ok && !mbar_wait_bounded(acc_empty + 8, accph, kWaitLimit)) ok = false;
+          tc_fence_after();
+          for (int kb = ke; kb < k1 && ok; ++kb) cross(true, 1u, kb != ke);  // phase M
+          if (!ok) break;
+          mma_commit_pair_mc(acc_full, 0x3);  // acc0 complete for this slab, both CTAs
+          if (square) {                       // phase B
+            for (int kb = k0; kb < ke && ok; ++kb) cross(false, 1u, ke < k1 || kb != k0);
+          } else {
+            for (int kb = k0; kb < ke && ok; ++kb) {
+              single(kAccCols, kb != k0);
+              if (ok) single(kAccCols, 1u);
+            }
+          }
+          if (!ok) break;
+          mma_commit_pair_mc(acc_full + 8, 0x3);
+          accph ^= 1;
+        }
+      }
+      if (!ok) {
+        ctx.dev->status = kStatusTimeout;
+        ctx.dev->timeout_site = 2;
+      }
+      // All MMAs retired before the tensor memory or the peer's shared memory goes away.
+      mma_commit_pair(drain_bar);
+      mbar_wait_bounded(drain_bar, 0, kWaitLimit);
+    }
+    __syncwarp();
+  } else {
+    // ---------------- epilogue (warps 2..17, both CTAs) ----------------
+    const int q = warp & 3;                    // TMEM lane quarter of this warp
+    const int h = (warp - 2) >> 2;             // 64-column quarter of the tile
+    const uint32_t lane_addr = tmem + (static_cast<uint32_t>(32 * q) << 16) + static_cast<uint32_t>(64 * h);
+    const uint32_t acc_empty_leader = mapa_shared(acc_empty, 0);
+    uint32_t accph = 0;
+    uint32_t pk[32];  // this thread's 64 running residues, two to a word
+    // Columns [c, c + 16) of accumulator a; after the last ones the
+    // accumulator is free.  The arrive is relaxed: a release would hold it
+    // until the residue stores before it are performed, and the MMAs need no
+    // ordering against those.
+    auto load16 = [&](int a, int c, uint32_t (&v)[16]) {
+      tmem_ld16(lane_addr + a * kAccCols + c, v);
+      tmem_ld_wait();
+      if (c == 48) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_remote_relaxed(acc_empty_leader + 8 * a);
+      }
+    };
+    for (int64_t w = 0, u = pair; u < um.nunits && ok; u = wave_unit(pair, ++w, npairs)) {
+      const Unit x = unit_at<0>(u, um);
+      const int i = x.i;
+      const int64_t row = x.tm * kTileM + rank * kRows + 32 * q + lane;
+      const int64_t col0 = x.tn * kTileN + 64 * h;
+      const bool square = mods.sq_base[i] != 0;
+      const float mf = static_cast<float>(mods.m[i]);
+      const float inv = 1.f / mf;
+      const float hi = static_cast<float>(mods.m[i] - 1 - mods.m[i] / 2);
+      // v = w0·acc0 + w1·acc1: acc0 + s·acc1 (Eq. sq-shortcut) or
+      // 16·acc0 - 15·acc1 (Eq. kar with the merged accumulator).
+      const float w0 = square ? 1.f : 16.f, w1 = square ? static_cast<float>(mods.sq_base[i]) : -15.f;
+      // This thread's row of C^(i) (of part `part` of it under split K);
+      // column j at rrow[j·ldr].
+      int16_t* rrow = ctx.res + (static_cast<size_t>(x.part) * mods.r + i) * ctx.n * ctx.ldr + row;
+      const int slab = residue_slab_steps(square), khi = static_cast<int>(x.k_hi);
+      for (int k0 = static_cast<int>(x.k_lo); k0 < khi; k0 += slab) {
+        const bool first = k0 == static_cast<int>(x.k_lo), last = k0 + slab >= khi;
+        // acc0, during phase B.  The first slab keeps a = acc0 mod m itself
+        // (|a| < 1.5m); a later one adds w0·a to the running residue
+        // (|w0·a| + m/2 < 2^14.1) and keeps that within 1.5m.
         if (!mbar_wait_bounded(acc_full, accph, kWaitLimit)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        // A slab other than the last leaves its centred residue r in the
-        // accumulators and the next slab accumulates on top of it: acc0 = r,
-        // acc1 = 0 for square moduli (v = acc0 + s·acc1), and acc0 = acc1 = r
-        // for nonsquare ones (16r - 15r = r).  The bounds of Eq. accum-exact
-        // keep their margin: 32768·256 + 544 and 4096·4095 + 255 < 2^24.
-        const bool carry = MODE == 0 && kb0 + slab < x.k_hi;
+#pragma unroll
         for (int c = 0; c < 64; c += 16) {
-          uint32_t v0[16], v1[16];
-          tmem_ld16(lane_addr + c, v0);
-          if (MODE == 0) tmem_ld16(lane_addr + kAccCols + c, v1);
-          tmem_ld_wait();
-          if (c == 48 && !carry) {
-            // The last chunk is in registers: release the accumulators now,
-            // so the next unit's MMAs overlap this chunk's reduction and
-            // stores.  The arrive is relaxed: the residue stores before it
-            // need no ordering against the MMAs, and a release would wait
-            // for them to be performed.
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_remote_relaxed(acc_empty_leader);
+          uint32_t v[16];
+          load16(0, c, v);
+#pragma unroll
+          for (int j = 0; j < 16; j += 2) {
+            float a[2];
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+              a[t] = loose_mod(__uint_as_float(v[j + t]), mf, inv);
+              if (!first) a[t] = loose_mod(fmaf(w0, a[t], unpack_scaled(pk[(c + j) / 2], t, 1.f)), mf, inv);
+            }
+            pk[(c + j) / 2] = pack_residues(a[0], a[1]);
           }
-          if (MODE == 1 && SHORT1) {  // a part of k: add this tile's partial sums into U
-            const int64_t cc = col0 + c;
-            if (row < ctx.m) {
-              float* dst = ctx.upart + row * ctx.ldu + cc;  // 16-byte aligned: ldu and cc multiples of 4
-              if (cc + 16 <= ctx.n) {
+        }
+        // acc1, during the next slab's or unit's phase A.  |v| ≤ 1.5m·(w0 +
+        // |w1|) < 2^16 (34·1.5·1089 for squares, 31·1.5·511 otherwise).
+        if (!mbar_wait_bounded(acc_full + 8, accph, kWaitLimit)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const float wp = first ? w0 : 1.f;
 #pragma unroll
-                for (int j = 0; j < 16; j += 4)
-                  atomicAdd(reinterpret_cast<float4*>(dst + j),
-                            make_float4(__uint_as_float(v0[j]), __uint_as_float(v0[j + 1]), __uint_as_float(v0[j + 2]),
-                                        __uint_as_float(v0[j + 3])));
-              } else {
+        for (int c = 0; c < 64; c += 16) {
+          uint32_t v[16];
+          load16(1, c, v);
+          const int64_t cc = col0 + c;
+          const int ncol = ctx.n - cc < 16 ? static_cast<int>(ctx.n - cc) : 16;
+          auto reduce = [&](int j) {
+            const float b = loose_mod(__uint_as_float(v[j]), mf, inv);
+            return centred_small(fmaf(w1, b, unpack_scaled(pk[(c + j) / 2], j & 1, wp)), mf, inv, hi);
+          };
+          if (!last) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j)
-                  if (cc + j < ctx.n) atomicAdd(dst + j, __uint_as_float(v0[j]));
-              }
+            for (int j = 0; j < 16; j += 2) {
+              const float r0 = reduce(j), r1 = reduce(j + 1);
+              pk[(c + j) / 2] = pack_residues(r0, r1);
             }
-          } else if (MODE == 1) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) rowmax = fmaxf(rowmax, __uint_as_float(v0[j]));
-          } else if (carry) {  // every lane: tcgen05.st is warp-collective
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const float rj =
-                  combine_residue(__uint_as_float(v0[j]), __uint_as_float(v1[j]), square, sb, mf, inv, hi, 0.f);
-              v0[j] = __float_as_uint(rj);
-              v1[j] = square ? 0u : v0[j];
-            }
-            tmem_st16(lane_addr + c, v0);
-            tmem_st16(lane_addr + kAccCols + c, v1);
           } else if (row < ctx.m) {
-            const int64_t cc = col0 + c;
             int16_t* dst = rrow + cc * ctx.ldr;
-            const int ncol = ctx.n - cc < 16 ? static_cast<int>(ctx.n - cc) : 16;
-            if (SHORT1 && ncol == 16 && square) {  // k ≤ 128: one short slab, every modulus
+            if (ncol == 16) {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const float rj =
-                    combine_residue_short1<true>(__uint_as_float(v0[j]), __uint_as_float(v1[j]), sb, mf, inv, hi);
-                *dst = static_cast<int16_t>(as_i16_bits(rj));
-                dst += ctx.ldr;
-              }
-            } else if (SHORT1 && ncol == 16) {
-#pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const float rj =
-                    combine_residue_short1<false>(__uint_as_float(v0[j]), __uint_as_float(v1[j]), sb, mf, inv, hi);
-                *dst = static_cast<int16_t>(as_i16_bits(rj));
-                dst += ctx.ldr;
-              }
-            } else if (!SHORT1 && ncol == 16 && short_slab) {  // a single short slab
-#pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const float rj =
-                    combine_residue_short(__uint_as_float(v0[j]), __uint_as_float(v1[j]), square, sb, mf, inv, hi);
-                *dst = static_cast<int16_t>(as_i16_bits(rj));
-                dst += ctx.ldr;
-              }
-            } else if (ncol == 16) {  // the common case: a full chunk
-#pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const float rj =
-                    combine_residue(__uint_as_float(v0[j]), __uint_as_float(v1[j]), square, sb, mf, inv, hi, 0.f);
-                *dst = static_cast<int16_t>(as_i16_bits(rj));
-                dst += ctx.ldr;
-              }
+              for (int j = 0; j < 16; ++j, dst += ctx.ldr) *dst = static_cast<int16_t>(as_i16_bits(reduce(j)));
             } else {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const float rj =
-                    combine_residue(__uint_as_float(v0[j]), __uint_as_float(v1[j]), square, sb, mf, inv, hi, 0.f);
-                if (j < ncol) dst[j * ctx.ldr] = static_cast<int16_t>(as_i16_bits(rj));
-              }
+              for (int j = 0; j < 16; ++j, dst += ctx.ldr)
+                if (j < ncol) *dst = static_cast<int16_t>(as_i16_bits(reduce(j)));
             }
           }
         }
-        if (carry) {  // the written-back residues are in place before the next slab's MMAs
-          tmem_st_wait();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_remote(acc_empty_leader);
-        }
         accph ^= 1;
-      }
-      if (MODE == 1 && !SHORT1 && ok) {
-        // rows past m hold zeros (TMA fills out-of-range rows with 0)
-        if (row < ctx.m) atomicMax(reinterpret_cast<int*>(ctx.urow) + row, __float_as_int(rowmax));
-        const int wm = __reduce_max_sync(0xffffffffu, __float_as_int(rowmax));
-        if (lane == 0) atomicMax(&ctx.dev->u_max_bits, wm);
       }
     }
     if (!ok) {
@@ -717,7 +1007,7 @@ int64_t residue_gemm_kparts(int64_t m, int64_t n, int64_t k_pad, int r, int nsq,
   return choose_kparts(ntiles, r, nsq, k_pad / kBK, pairs, m, n, max_parts);
 }
 
-static size_t gemm_smem_bytes() { return 1024 + static_cast<size_t>(kStages) * kStageBytes + 8 * (2 * kStages + 3); }
+static size_t gemm_smem_bytes() { return 1024 + static_cast<size_t>(kStages) * kStageBytes + 8 * (2 * kStages + 5); }
 
 // The magnitude GEMM split along k: each part adds its tiles' partial sums
 // into U with 16-byte vector atomics (every partial sum is an integer number
@@ -797,7 +1087,7 @@ cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Modu
   um.kparts = 1;
   um.kpart_steps = um.ksteps;
   const size_t smem = gemm_smem_bytes();
-  auto kern = mode == 1 ? plane_gemm_kernel<1> : k_pad == kBK ? plane_gemm_kernel<0, true> : plane_gemm_kernel<0>;
+  auto kern = mode == 1 ? plane_gemm_kernel<1> : k_pad == kBK ? plane_gemm_kernel<0> : residue_gemm_kernel;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (err != cudaSuccess) return err;
   // Persistent grid: as many CTA pairs as can be resident at once.

@@ -48,24 +48,20 @@ __device__ __forceinline__ float combine_residue(float a0, float a1, bool square
   const float v = (square ? fmaf(s, r1, r0) : fmaf(16.f, r0, -15.f * r1)) + prev;
   return centred_small(v, m, inv_m, hi);
 }
-// The same for a short slab, where v itself is an integer below 2^24 and the
-// accumulators need no reduction before they are combined (see short_slab).
-__device__ __forceinline__ float combine_residue_short(float a0, float a1, bool square, float s, float m,
-                                                       float inv_m, float hi) {
-  const float v = square ? fmaf(s, a1, a0) : fmaf(16.f, a0, -15.f * a1);
-  return centred_small(loose_mod(v, m, inv_m), m, inv_m, hi);
-}
-// The short-K kernel's form (k ≤ 128, one k-block): loose_mod leaves r with
-// |r| < 1.5m, so one step toward the centred range [hi + 1 - m, hi] finishes
-// (above hi, r - m ≥ hi + 1 - m; below it, r + m ≤ hi), and SQUARE, uniform
-// over a unit, is a template parameter.
-template <bool SQUARE>
-__device__ __forceinline__ float combine_residue_short1(float a0, float a1, float s, float m, float inv_m,
-                                                        float hi) {
-  const float v = SQUARE ? fmaf(s, a1, a0) : fmaf(16.f, a0, -15.f * a1);
+// The form for k ≤ 128 (one k-block), where the recombined v itself is an
+// integer below 2^24 (|v| ≤ 128·(256 + 33·512) for squares, 128·(16·484 +
+// 15·4095) otherwise): loose_mod leaves r with |r| < 1.5m, so one step toward
+// the centred range [hi + 1 - m, hi] finishes (above hi, r - m ≥ hi + 1 - m;
+// below it, r + m ≤ hi).
+__device__ __forceinline__ float short_residue(float v, float m, float inv_m, float hi) {
   float r = loose_mod(v, m, inv_m);
   r = r > hi ? r - m : r;
   return r < hi + 1.f - m ? r + m : r;
+}
+template <bool SQUARE>
+__device__ __forceinline__ float combine_residue_short1(float a0, float a1, float s, float m, float inv_m,
+                                                        float hi) {
+  return short_residue(SQUARE ? fmaf(s, a1, a0) : fmaf(16.f, a0, -15.f * a1), m, inv_m, hi);
 }
 // int16 encoding of an integer-valued float in [-2^15, 2^15).
 __device__ __forceinline__ uint32_t as_i16_bits(float r) { return __float_as_uint(r + kRoundMagic) & 0xFFFFu; }
