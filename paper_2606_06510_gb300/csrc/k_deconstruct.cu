@@ -306,25 +306,38 @@ template <int MODE, int R>
 __global__ void __launch_bounds__(TileShape<MODE>::kThreads, TileShape<MODE>::kBlocksPerSm) planes_kernel(OperandView X0, OperandView X1, int blocks0, int64_t k,
                                                              int64_t k_pad, int clamp_c, int rn,
                                                              const __grid_constant__ Oz2Moduli mods) {
-  extern __shared__ uint32_t table[];
+  extern __shared__ __align__(16) uint32_t table[];
   const bool second = static_cast<int>(blockIdx.x) >= blocks0;
   const OperandView X = second ? X1 : X0;
   const int bid = second ? blockIdx.x - blocks0 : blockIdx.x;
   const int nblocks = second ? gridDim.x - blocks0 : blocks0;
-  if (MODE == 1) {
-    for (int t = threadIdx.x; t < mods.table_entries; t += blockDim.x) table[t] = X.table[t];
-    __syncthreads();
-  }
   using TS = TileShape<MODE>;
+  const int tile_rows = blockDim.x / TS::kThreadsPerRow;
   const int64_t rows_out = rows_stored<MODE>(X.rows);
-  const int64_t row_tiles = (rows_out + TS::kRows - 1) / TS::kRows;
+  const int64_t row_tiles = (rows_out + tile_rows - 1) / tile_rows;
   const int64_t ntiles = row_tiles * (k_pad / TS::kSeg);
   const int part = threadIdx.x & (TS::kThreadsPerRow - 1);
   const int rloc = threadIdx.x / TS::kThreadsPerRow;
+  if (MODE == 1) {
+    // The block's copy of the table, 16 bytes a load and four loads in flight
+    // (word by word the copy alone took 6 µs of a one-tile block's time).
+    const uint4* src = reinterpret_cast<const uint4*>(X.table);
+    const int words4 = (mods.table_entries + 3) >> 2;
+    for (int t0 = threadIdx.x; t0 < words4; t0 += 4 * blockDim.x) {
+      uint4 v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (t0 + j * blockDim.x < words4) v[j] = __ldg(src + t0 + j * blockDim.x);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (t0 + j * blockDim.x < words4) reinterpret_cast<uint4*>(table)[t0 + j * blockDim.x] = v[j];
+    }
+    __syncthreads();
+  }
 
   for (int64_t tile = bid; tile < ntiles; tile += nblocks) {
     const int64_t kt = tile / row_tiles;  // consecutive blocks share a k-slice of many rows
-    const int64_t row = (tile - kt * row_tiles) * TS::kRows + rloc;
+    const int64_t row = (tile - kt * row_tiles) * tile_rows + rloc;
     if (row >= rows_out) continue;
     const int64_t l0 = kt * TS::kSeg + part * kElems;
     const bool pad = row >= X.rows;  // pad rows of the last block: zero digits
@@ -771,12 +784,23 @@ cudaError_t launch_deconstruct(int64_t m, int64_t n, int64_t k, const Oz2Moduli&
                                const uint8_t* row_flag, const uint8_t* col_flag, int quant,
                                uint8_t* planes_a, uint8_t* planes_b, cudaStream_t st) {
   const int64_t k_pad = (k + kKPad - 1) / kKPad * kKPad;
-  const size_t smem = sizeof(uint32_t) * mods.table_entries;
+  const size_t smem = sizeof(uint32_t) * ((mods.table_entries + 3) & ~3);  // copied in 16-byte words
   const int rn = quant == OZ2_QUANT_RN;
   OperandView va{A, 1, lda, m, d, row_flag, planes_a, table_a, 0};
   OperandView vb{B, ldb, 1, n, e, col_flag, planes_b, table_b, vec_ok(B, ldb, 1)};
+  // A small problem has fewer full tiles than the GPU has SMs: its blocks then
+  // take a quarter of the rows each (256³: 32 tiles of 32 rows on 152 SMs,
+  // 14.8 µs, against 128 of 8 rows, 7.5).
+  int threads = TileShape<1>::kThreads, per_sm = TileShape<1>::kBlocksPerSm;
+  int64_t t0 = m ? tiles_of<1>(m, k_pad) : 0, t1 = n ? tiles_of<1>(n, k_pad) : 0;
+  if (t0 + t1 <= num_sms()) {
+    threads /= 4;
+    per_sm *= 4;
+    t0 *= 4;
+    t1 *= 4;
+  }
   int g0, g1;
-  split_grid(m ? tiles_of<1>(m, k_pad) : 0, n ? tiles_of<1>(n, k_pad) : 0, TileShape<1>::kBlocksPerSm, &g0, &g1);
+  split_grid(t0, t1, per_sm, &g0, &g1);
   if (g0 + g1 == 0) return cudaSuccess;
   if (g0 == 0) va = vb;
   cudaError_t err = cudaSuccess;
@@ -787,7 +811,7 @@ cudaError_t launch_deconstruct(int64_t m, int64_t n, int64_t k, const Oz2Moduli&
     err = cudaFuncSetAttribute(planes_kernel<1, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,            \
                                static_cast<int>(smem));                                                     \
     if (err == cudaSuccess)                                                                                 \
-      planes_kernel<1, R><<<g0 + g1, TileShape<1>::kThreads, smem, st>>>(va, vb, g0, k, k_pad, 0, rn, mods); \
+      planes_kernel<1, R><<<g0 + g1, threads, smem, st>>>(va, vb, g0, k, k_pad, 0, rn, mods); \
     break;
     OZ2_DEC_CASE(1) OZ2_DEC_CASE(2) OZ2_DEC_CASE(3) OZ2_DEC_CASE(4) OZ2_DEC_CASE(5) OZ2_DEC_CASE(6)
     OZ2_DEC_CASE(7) OZ2_DEC_CASE(8) OZ2_DEC_CASE(9) OZ2_DEC_CASE(10) OZ2_DEC_CASE(11) OZ2_DEC_CASE(12)

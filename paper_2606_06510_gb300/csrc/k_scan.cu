@@ -4,6 +4,7 @@
 #include <climits>
 
 #include "k_scan.cuh"
+#include "oz2_gemm.cuh"
 
 namespace oz2 {
 
@@ -35,9 +36,12 @@ __device__ __forceinline__ void scan_a_rows(int64_t bx, int64_t by, int64_t m, i
   int best = 0;
   const double* p = A + i + l0 * lda;
   int64_t l = l0;
-  for (; l + 4 <= l1; l += 4, p += 4 * lda) {
-    double x0 = __ldg(p), x1 = __ldg(p + lda), x2 = __ldg(p + 2 * lda), x3 = __ldg(p + 3 * lda);
-    best = max(best, max(max(scan_key(x0), scan_key(x1)), max(scan_key(x2), scan_key(x3))));
+  for (; l + 8 <= l1; l += 8, p += 8 * lda) {  // eight loads in flight
+    double x[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) x[j] = __ldg(p + j * lda);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) best = max(best, scan_key(x[j]));
   }
   for (; l < l1; ++l, p += lda) best = max(best, scan_key(__ldg(p)));
   if (best) atomicMax(key + i, best);
@@ -59,22 +63,23 @@ __device__ __forceinline__ void scan_b_cols(int64_t bx, int64_t by, int64_t n, i
     const double2* c2 = reinterpret_cast<const double2*>(col);
     const int64_t p1 = l1 >> 1;  // pairs fully inside [l0, l1) (l0 is even)
     int64_t p = (l0 >> 1) + lane;
-    for (; p + 96 < p1; p += 128) {
-      const double2 a = __ldg(c2 + p), b = __ldg(c2 + p + 32), c = __ldg(c2 + p + 64), d = __ldg(c2 + p + 96);
-      best = max(best, max(max(max(scan_key(a.x), scan_key(a.y)), max(scan_key(b.x), scan_key(b.y))),
-                           max(max(scan_key(c.x), scan_key(c.y)), max(scan_key(d.x), scan_key(d.y)))));
-    }
-    for (; p < p1; p += 32) {
-      const double2 a = __ldg(c2 + p);
-      best = max(best, max(scan_key(a.x), scan_key(a.y)));
+    for (; p < p1; p += 128) {  // four loads in flight, the last step's too
+      double2 a[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) a[j] = p + 32 * j < p1 ? __ldg(c2 + p + 32 * j) : make_double2(0.0, 0.0);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) best = max(best, max(scan_key(a[j].x), scan_key(a[j].y)));
     }
     if ((l1 & 1) && lane == 0) best = max(best, scan_key(__ldg(col + l1 - 1)));
   } else {
     int64_t l = l0 + lane;
-    for (; l + 96 < l1; l += 128)
-      best = max(best, max(max(scan_key(__ldg(col + l)), scan_key(__ldg(col + l + 32))),
-                           max(scan_key(__ldg(col + l + 64)), scan_key(__ldg(col + l + 96)))));
-    for (; l < l1; l += 32) best = max(best, scan_key(__ldg(col + l)));
+    for (; l < l1; l += 128) {
+      double a[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) a[j] = l + 32 * j < l1 ? __ldg(col + l + 32 * j) : 0.0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) best = max(best, scan_key(a[j]));
+    }
   }
   best = __reduce_max_sync(0xffffffffu, best);
   if (lane == 0 && best) atomicMax(key + j, best);
@@ -125,9 +130,16 @@ __global__ void __launch_bounds__(kFinalizeThreads) finalize_flags_kernel(int64_
   for (int b = threadIdx.x; b < kExpBins; b += blockDim.x) hist[b] = 0;
   if (threadIdx.x == 0) count_s = 0;
   __syncthreads();
-  for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x) {
-    int kv = key[i];
-    if (kv > 0 && kv < (1 << 20)) atomicAdd(&hist[kv - 2048 + kExpBias], 1);
+  // Keys in batches of eight independent loads: one block reads them all, so
+  // their latency is what this kernel takes for a large operand.
+  constexpr int kBatch = 8;
+  for (int64_t i0 = threadIdx.x; i0 < cnt; i0 += kBatch * kFinalizeThreads) {
+    int kv[kBatch];
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) kv[j] = i0 + j * kFinalizeThreads < cnt ? key[i0 + j * kFinalizeThreads] : 0;
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j)
+      if (kv[j] > 0 && kv[j] < (1 << 20)) atomicAdd(&hist[kv[j] - 2048 + kExpBias], 1);
   }
   __syncthreads();
   // Lower median of the histogram: each thread sums kBinsPerThread bins, a
@@ -179,16 +191,23 @@ __global__ void __launch_bounds__(kFinalizeThreads) finalize_flags_kernel(int64_
   const int med = med_s;
   const bool window = (flags & OZ2_FLAG_NO_FALLBACK) == 0;
   int local = 0;
-  for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x) {
-    int kv = key[i];
-    bool nonfinite = kv >= (1 << 20);
-    bool nonzero = kv > 0 && !nonfinite;
-    int e = nonzero ? kv - 2048 : 0;
-    bool fb = nonfinite || (window && nonzero && abs(e - med) > kFallbackWindow);
-    bool zero = fb || !nonzero;
-    fl[i] = static_cast<uint8_t>((fb ? 1 : 0) | (zero ? 2 : 0));
-    key[i] = zero ? 0 : e;
-    local += fb ? 1 : 0;
+  for (int64_t i0 = threadIdx.x; i0 < cnt; i0 += kBatch * kFinalizeThreads) {
+    int kv[kBatch];
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) kv[j] = i0 + j * kFinalizeThreads < cnt ? key[i0 + j * kFinalizeThreads] : 0;
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) {
+      const int64_t i = i0 + j * kFinalizeThreads;
+      if (i >= cnt) break;
+      const bool nonfinite = kv[j] >= (1 << 20);
+      const bool nonzero = kv[j] > 0 && !nonfinite;
+      const int e = nonzero ? kv[j] - 2048 : 0;
+      const bool fb = nonfinite || (window && nonzero && abs(e - med) > kFallbackWindow);
+      const bool zero = fb || !nonzero;
+      fl[i] = static_cast<uint8_t>((fb ? 1 : 0) | (zero ? 2 : 0));
+      key[i] = zero ? 0 : e;
+      local += fb ? 1 : 0;
+    }
   }
   if (local) atomicAdd(&count_s, local);
   __syncthreads();
@@ -202,21 +221,27 @@ cudaError_t launch_scan_keys(int64_t m, int64_t n, int64_t k, const double* A, i
                              int64_t ldb, ScanOut out, cudaStream_t st) {
   if (k <= 0 || (m <= 0 && n <= 0)) return cudaSuccess;
   ScanGrid g{};
+  // Rows of A: 64 k-entries per thread when that makes enough blocks to fill
+  // the GPU (eight of 256 threads per SM), shorter runs down to 8 (one batch
+  // of loads) when it does not: a small operand's scan is the latency of one
+  // thread's run (256³: 64 entries 13.7 µs, 8 entries 3.2).
+  g.gax = (m + 255) / 256;
   g.achunk = 64;
+  while (g.achunk > 8 && g.gax * ((k + g.achunk - 1) / g.achunk) < 8 * num_sms()) g.achunk /= 2;
   int64_t ks = (k + g.achunk - 1) / g.achunk;
   if (ks > 65535) {
     g.achunk = static_cast<int>((k + 65534) / 65535);
     ks = (k + g.achunk - 1) / g.achunk;
   }
-  g.bchunk = 1024;
+  // Columns of B: 1024 entries per warp, or one batch of loads (256) alike.
+  g.gbx = (n + 7) / 8;
+  g.bchunk = g.gbx * ((k + 1023) / 1024) < 8 * num_sms() ? 256 : 1024;
   int64_t bks = (k + g.bchunk - 1) / g.bchunk;
   if (bks > 65535) {
     g.bchunk = static_cast<int>((k + 65534) / 65535 + 1) & ~1;
     bks = (k + g.bchunk - 1) / g.bchunk;
   }
-  g.gax = (m + 255) / 256;
   g.ga = m > 0 ? g.gax * ks : 0;
-  g.gbx = (n + 7) / 8;
   const int64_t gb = n > 0 ? g.gbx * bks : 0;
   g.vec = (ldb % 2 == 0) && (reinterpret_cast<uintptr_t>(B) % 16 == 0);
   if (g.ga + gb > 0x7FFFFFFFLL) return cudaErrorInvalidValue;

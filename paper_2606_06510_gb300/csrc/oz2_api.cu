@@ -27,7 +27,7 @@ constexpr int kHostAChunksMax = 4;  // column chunks A is copied in by oz2_dgemm
 // nonsquare moduli, 2m entries per modulus, entry i for the residue
 // (i - kDecBias) mod m; table 0 for A (last plane pre-scaled by -16), table 1
 // for B.
-static __device__ uint32_t g_plane_table[2][kTableMax];
+static __device__ __align__(16) uint32_t g_plane_table[2][kTableMax];  // copied in 16-byte words
 // Device status block (sticky status word, fallback counts, scale summary).
 static __device__ Oz2Device g_status;
 
