@@ -131,6 +131,8 @@ __global__ void __launch_bounds__(kCrtThreads, crt_min_blocks<R, FAST>())
     crt_kernel(int64_t row0, int64_t rows, int64_t n, const __grid_constant__ Oz2Moduli mods,
                const int16_t* __restrict__ res, int64_t ldr, const int* __restrict__ d, const int* __restrict__ e,
                double* __restrict__ C, int64_t ldc) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t rel = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) * 2;
   if (rel >= rows) return;
   const int64_t row = row0 + rel;
@@ -175,9 +177,8 @@ static cudaError_t launch_crt_rows(cudaStream_t st, int64_t row0, int64_t rows, 
   gy = gy > n ? n : gy;
   gy = gy > 65535 ? 65535 : gy;
   count_launch();
-  crt_kernel<R, FAST><<<dim3(static_cast<unsigned>(gx), static_cast<unsigned>(gy)), kCrtThreads, 0, st>>>(
-      row0, rows, n, mods, res, ldr, d, e, C, ldc);
-  return cudaGetLastError();
+  return launch_dependent(crt_kernel<R, FAST>, dim3(static_cast<unsigned>(gx), static_cast<unsigned>(gy)),
+                          dim3(kCrtThreads), 0, st, row0, rows, n, mods, res, ldr, d, e, C, ldc);
 }
 
 template <int R>

@@ -307,6 +307,7 @@ __global__ void __launch_bounds__(TileShape<MODE>::kThreads, TileShape<MODE>::kB
                                                              int64_t k_pad, int clamp_c, int rn,
                                                              const __grid_constant__ Oz2Moduli mods) {
   extern __shared__ __align__(16) uint32_t table[];
+  pdl_trigger();
   const bool second = static_cast<int>(blockIdx.x) >= blocks0;
   const OperandView X = second ? X1 : X0;
   const int bid = second ? blockIdx.x - blocks0 : blockIdx.x;
@@ -334,6 +335,7 @@ __global__ void __launch_bounds__(TileShape<MODE>::kThreads, TileShape<MODE>::kB
     }
     __syncthreads();
   }
+  pdl_wait();  // exponents and flags; the table is constant
 
   for (int64_t tile = bid; tile < ntiles; tile += nblocks) {
     const int64_t kt = tile / row_tiles;  // consecutive blocks share a k-slice of many rows
@@ -774,8 +776,8 @@ cudaError_t launch_magnitude_planes(int64_t m, int64_t n, int64_t k, const doubl
   if (g0 + g1 == 0) return cudaSuccess;
   if (g0 == 0) va = vb;
   count_launch();
-  planes_kernel<0, 0><<<g0 + g1, TileShape<0>::kThreads, 0, st>>>(va, vb, g0, k, k_pad, c, 0, dummy);
-  return cudaGetLastError();
+  return launch_dependent(planes_kernel<0, 0>, dim3(g0 + g1), dim3(TileShape<0>::kThreads), 0, st, va, vb, g0, k, k_pad,
+                          c, 0, dummy);
 }
 
 cudaError_t launch_deconstruct(int64_t m, int64_t n, int64_t k, const Oz2Moduli& mods,
@@ -811,7 +813,8 @@ cudaError_t launch_deconstruct(int64_t m, int64_t n, int64_t k, const Oz2Moduli&
     err = cudaFuncSetAttribute(planes_kernel<1, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,            \
                                static_cast<int>(smem));                                                     \
     if (err == cudaSuccess)                                                                                 \
-      planes_kernel<1, R><<<g0 + g1, threads, smem, st>>>(va, vb, g0, k, k_pad, 0, rn, mods); \
+      err = launch_dependent(planes_kernel<1, R>, dim3(g0 + g1), dim3(threads), smem, st, va, vb, g0, k, k_pad, 0, \
+                             rn, mods);                                                                     \
     break;
     OZ2_DEC_CASE(1) OZ2_DEC_CASE(2) OZ2_DEC_CASE(3) OZ2_DEC_CASE(4) OZ2_DEC_CASE(5) OZ2_DEC_CASE(6)
     OZ2_DEC_CASE(7) OZ2_DEC_CASE(8) OZ2_DEC_CASE(9) OZ2_DEC_CASE(10) OZ2_DEC_CASE(11) OZ2_DEC_CASE(12)

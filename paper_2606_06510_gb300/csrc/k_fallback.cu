@@ -19,6 +19,8 @@ constexpr int kFT = 64, kFK = 16;
 __global__ void compact_flags_kernel(int64_t m, int64_t n, const uint8_t* __restrict__ row_flag,
                                      const uint8_t* __restrict__ col_flag, int* __restrict__ row_list,
                                      int* __restrict__ col_list, int* __restrict__ count) {
+  pdl_trigger();
+  pdl_wait();
   const bool cols = blockIdx.y == 1;
   const int64_t cnt = cols ? n : m;
   const uint8_t* flag = cols ? col_flag : row_flag;
@@ -132,7 +134,9 @@ cudaError_t launch_fallback_lists(int64_t m, int64_t n, int64_t k, const double*
   count_launch(2);
   const int64_t most = m > n ? m : n;
   const unsigned cg = static_cast<unsigned>(std::min<int64_t>((most + 255) / 256, 4096));
-  compact_flags_kernel<<<dim3(cg, 2), 256, 0, st>>>(m, n, row_flag, col_flag, rlist, clist, counts);
+  const cudaError_t err =
+      launch_dependent(compact_flags_kernel, dim3(cg, 2), dim3(256), 0, st, m, n, row_flag, col_flag, rlist, clist, counts);
+  if (err != cudaSuccess) return err;
   // flagged rows × all columns (blockIdx.y = 0), all rows × flagged columns (1)
   fma_gemm_kernel<<<dim3(fb_grid(), 2), 256, 0, st>>>(m, n, k, A, lda, B, ldb, rlist, counts, clist, counts + 1, C,
                                                        ldc);

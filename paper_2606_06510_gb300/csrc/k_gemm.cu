@@ -168,6 +168,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
   bool ok = true;
+  pdl_wait();  // the planes are written; the set-up above overlaps that kernel's tail
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
@@ -498,6 +499,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
   bool ok = true;
+  pdl_wait();  // the planes are written; the set-up above overlaps that kernel's tail
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
@@ -896,6 +898,7 @@ __global__ void __launch_bounds__(kFoldThreads) fold_parts_kernel(const int16_t*
                                                                   int16_t* __restrict__ res, int64_t m, int64_t n,
                                                                   int64_t ldr, int kparts,
                                                                   const __grid_constant__ Oz2Moduli mods) {
+  pdl_wait();
   const int i = blockIdx.z;
   const float mf = static_cast<float>(mods.m[i]), inv = 1.f / mf;
   const float hi = static_cast<float>(mods.m[i] - 1 - mods.m[i] / 2);
@@ -1018,6 +1021,7 @@ constexpr int kRowMaxThreads = 256;
 __global__ void __launch_bounds__(kRowMaxThreads) plus_one_rowmax_kernel(const float* __restrict__ U, int64_t m,
                                                                          int64_t n, int64_t ldu,
                                                                          float* __restrict__ urow, Oz2Device* dev) {
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int64_t row = static_cast<int64_t>(blockIdx.x) * (kRowMaxThreads / 32) + (threadIdx.x >> 5);
   if (row >= m) return;  // whole warps
@@ -1138,21 +1142,27 @@ cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Modu
   }
   pairs = std::max<int64_t>(1, std::min<int64_t>(pairs, um.nunits));
   count_launch();
-  kern<<<static_cast<unsigned>(2 * pairs), kGemmThreads, smem, st>>>(ta, tb, mods, k_pad, um, ctx);
-  if (ctx.upart) {
+  // The GEMM kernels let no dependent start early: the deconstruction's two
+  // blocks per SM, resident beside the "+1" GEMM on the SMs it leaves room on,
+  // spread unevenly (16384×16×16384 4172 µs a call, 4408 with the early start;
+  // 1024²×65536 2795 and 2873).
+  err = launch_dependent(kern, dim3(static_cast<unsigned>(2 * pairs)), dim3(kGemmThreads), smem, st, ta, tb, mods, k_pad,
+                         um, ctx);
+  if (err == cudaSuccess && ctx.upart) {
     count_launch();
     constexpr int64_t rows_per_block = kRowMaxThreads / 32;
-    plus_one_rowmax_kernel<<<static_cast<unsigned>((m + rows_per_block - 1) / rows_per_block), kRowMaxThreads, 0,
-                             st>>>(ctx.upart, m, n, ctx.ldu, urow, dev);
+    err = launch_dependent(plus_one_rowmax_kernel, dim3(static_cast<unsigned>((m + rows_per_block - 1) / rows_per_block)),
+                           dim3(kRowMaxThreads), 0, st, ctx.upart, m, n, ctx.ldu, urow, dev);
   }
-  if (mode == 0 && um.kparts > 1) {  // the residue GEMM's parts, folded into C^(i)
+  if (err == cudaSuccess && mode == 0 && um.kparts > 1) {  // the residue GEMM's parts, folded into C^(i)
     const int64_t row_threads = (m + 7) / 8;
     dim3 g(static_cast<unsigned>((row_threads + kFoldThreads - 1) / kFoldThreads),
            static_cast<unsigned>(std::min<int64_t>(n, 32768)), static_cast<unsigned>(mods.r));
     count_launch();
-    fold_parts_kernel<<<g, kFoldThreads, 0, st>>>(partials, residues, m, n, ldr, static_cast<int>(um.kparts), mods);
+    err = launch_dependent(fold_parts_kernel, g, dim3(kFoldThreads), 0, st, partials, residues, m, n, ldr, um.kparts,
+                           mods);
   }
-  return cudaGetLastError();
+  return err;
 }
 
 // The rate probe on as many CTA pairs as can be resident at once.

@@ -44,6 +44,7 @@ __device__ __forceinline__ void scan_a_rows(int64_t bx, int64_t by, int64_t m, i
     for (int j = 0; j < 8; ++j) best = max(best, scan_key(x[j]));
   }
   for (; l < l1; ++l, p += lda) best = max(best, scan_key(__ldg(p)));
+  pdl_wait();  // the keys are zeroed (the operands were complete before that launch)
   if (best) atomicMax(key + i, best);
 }
 
@@ -82,6 +83,7 @@ __device__ __forceinline__ void scan_b_cols(int64_t bx, int64_t by, int64_t n, i
     }
   }
   best = __reduce_max_sync(0xffffffffu, best);
+  pdl_wait();
   if (lane == 0 && best) atomicMax(key + j, best);
 }
 
@@ -122,6 +124,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) finalize_flags_kernel(int64_
   __shared__ int warp_sum[32];
   __shared__ int med_s;
   __shared__ int count_s;
+  pdl_trigger();
   pdl_wait();  // the scan keys are complete
   const bool is_a = blockIdx.x + first_op == 0;
   const int64_t cnt = is_a ? m : n;
@@ -218,7 +221,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) finalize_flags_kernel(int64_
 }
 
 cudaError_t launch_scan_keys(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
-                             int64_t ldb, ScanOut out, cudaStream_t st) {
+                             int64_t ldb, ScanOut out, cudaStream_t st, bool dependent) {
   if (k <= 0 || (m <= 0 && n <= 0)) return cudaSuccess;
   ScanGrid g{};
   // Rows of A: 64 k-entries per thread when that makes enough blocks to fill
@@ -246,7 +249,13 @@ cudaError_t launch_scan_keys(int64_t m, int64_t n, int64_t k, const double* A, i
   g.vec = (ldb % 2 == 0) && (reinterpret_cast<uintptr_t>(B) % 16 == 0);
   if (g.ga + gb > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
   count_launch();
-  scan_kernel<<<static_cast<unsigned>(g.ga + gb), 256, 0, st>>>(m, n, k, A, lda, B, ldb, g, out.ra, out.cb);
+  // As a dependent of the kernel that zeroes the keys, the scan reads the
+  // operands while that kernel runs; it must not where the operands are still
+  // arriving, so the caller says (`dependent`).
+  const dim3 grid(static_cast<unsigned>(g.ga + gb));
+  if (dependent)
+    return launch_dependent(scan_kernel, grid, dim3(256), 0, st, m, n, k, A, lda, B, ldb, g, out.ra, out.cb);
+  scan_kernel<<<grid, 256, 0, st>>>(m, n, k, A, lda, B, ldb, g, out.ra, out.cb);
   return cudaGetLastError();
 }
 
@@ -268,7 +277,7 @@ cudaError_t launch_scan(int64_t m, int64_t n, int64_t k, const double* A, int64_
   // The scan keys are maxima taken with atomics: zero unless the caller has.
   if (zero_keys && m > 0 && (err = cudaMemsetAsync(out.ra, 0, sizeof(int) * m, st)) != cudaSuccess) return err;
   if (zero_keys && n > 0 && (err = cudaMemsetAsync(out.cb, 0, sizeof(int) * n, st)) != cudaSuccess) return err;
-  if ((err = launch_scan_keys(m, n, k, A, lda, B, ldb, out, st)) != cudaSuccess) return err;
+  if ((err = launch_scan_keys(m, n, k, A, lda, B, ldb, out, st, !zero_keys)) != cudaSuccess) return err;
   return launch_scan_flags(m, n, 3, flags, out, dev, st);
 }
 
@@ -288,6 +297,8 @@ __global__ void choose_scales_kernel(int64_t m, int64_t n, int64_t k, int T, int
                                      const uint8_t* __restrict__ row_flag,
                                      const uint8_t* __restrict__ col_flag, int* __restrict__ d,
                                      int* __restrict__ e, Oz2Device* dev) {
+  pdl_trigger();
+  pdl_wait();
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   int s, umax = 0;
   if (scale_mode == OZ2_SCALE_R2) {
@@ -327,9 +338,8 @@ cudaError_t launch_choose_scales(int64_t m, int64_t n, int64_t k, const Oz2Modul
   int64_t tot = m + n;
   if (tot == 0) return cudaSuccess;
   count_launch();
-  choose_scales_kernel<<<static_cast<unsigned>((tot + 255) / 256), 256, 0, st>>>(
-      m, n, k, mods.T, scale_mode, urow, ra, cb, row_flag, col_flag, d, e, dev);
-  return cudaGetLastError();
+  return launch_dependent(choose_scales_kernel, dim3(static_cast<unsigned>((tot + 255) / 256)), dim3(256), 0, st, m, n,
+                          k, mods.T, scale_mode, urow, ra, cb, row_flag, col_flag, d, e, dev);
 }
 
 }  // namespace oz2

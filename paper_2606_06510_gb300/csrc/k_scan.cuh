@@ -11,9 +11,11 @@ namespace oz2 {
 // lda) and of the columns of B (k × n at B, leading dimension ldb), merged
 // into out.ra and out.cb by atomic maximum, so a column chunk of A
 // (A + k0·lda with k its width) merges into the same row keys as the rest.
-// m or n may be 0 to scan one operand only.  The keys must be zeroed first.
+// m or n may be 0 to scan one operand only.  The keys must be zeroed first;
+// with `dependent`, by the kernel launched just before, which itself started
+// after the operands were complete (the scan then reads them while it runs).
 cudaError_t launch_scan_keys(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
-                             int64_t ldb, ScanOut out, cudaStream_t st);
+                             int64_t ldb, ScanOut out, cudaStream_t st, bool dependent = false);
 
 // Fallback flags and final exponents from complete keys: A's rows when
 // ops & 1, B's columns when ops & 2.  Launched as a programmatic dependent

@@ -382,6 +382,7 @@ __global__ void reset_status_kernel(Oz2Device* dev) {
 // maxima; the two fallback counts) set to zero, in one launch.
 __global__ void prepare_call_kernel(Oz2Device* dev, int* ra, int64_t m, int* cb, int64_t n, float* urow,
                                     int* counts) {
+  pdl_trigger();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     dev->fallback_rows = 0;
     dev->fallback_cols = 0;
