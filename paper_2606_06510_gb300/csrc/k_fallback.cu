@@ -6,6 +6,11 @@
 // Tiled CUDA-core DGEMM over index lists: 64×64 output tiles, 256 threads,
 // 4×4 outputs per thread, k staged through shared memory in chunks of 16.
 // The same kernel is the cuBLAS-free native comparator (identity lists).
+//
+// The FP64 pipe bounds it (two FMAs a cycle per SM): the next chunk's entries
+// are fetched while one is multiplied, B's along k, and rows past the list's
+// end multiply nothing (164 flagged rows of 16384²×64: 0.404 → 0.371 ms, 0.28
+// at that rate).
 #include <algorithm>
 
 #include "oz2_common.cuh"
@@ -70,22 +75,34 @@ __global__ void __launch_bounds__(256) fma_gemm_kernel(int64_t m, int64_t n, int
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
+    // A chunk's entries are in registers one chunk ahead.  A: a thread's four
+    // lie in one row (row t mod 64, k t/64 + 4q); B: k fastest, 16 lanes on
+    // 128 consecutive bytes of a column (column t/16 + 16q, k t mod 16).
+    const int ar = threadIdx.x & 63, ak = threadIdx.x >> 6, bc = threadIdx.x >> 4, bk = threadIdx.x & 15;
+    double fa[4], fb[4];
+    auto fetch = [&](int64_t l0) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int gi = rid[ar], gj = cid[bc + 16 * q];
+        const int64_t la = l0 + ak + 4 * q, lb = l0 + bk;
+        fa[q] = (gi >= 0 && la < k) ? A[gi + la * lda] : 0.0;
+        fb[q] = (gj >= 0 && lb < k) ? B[lb + gj * ldb] : 0.0;
+      }
+    };
+    // Rows and columns past the lists' ends cost no FP64 work: the pipe is
+    // what bounds this kernel (2 FMAs a cycle per SM).
+    const bool live = rid[ty * 4] >= 0 && cid[tx * 4] >= 0;
+    if (k > 0) fetch(0);
     for (int64_t l0 = 0; l0 < k; l0 += kFK) {
       __syncthreads();
-      // A tile: 64 rows × 16 k; thread loads 4 entries (row = t % 64, k = t / 64 + 4q).
+#pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int rr = threadIdx.x & 63, kk = (threadIdx.x >> 6) + 4 * q;
-        const int gi = rid[rr];
-        const int64_t l = l0 + kk;
-        As[kk][rr] = (gi >= 0 && l < k) ? A[gi + l * lda] : 0.0;
-        const int cc = threadIdx.x & 63;
-        const int gj = cid[cc];
-        // B tile: 16 k × 64 cols; same pattern (k fastest would coalesce better;
-        // the fallback is rare and small).
-        Bs[kk][cc] = (gj >= 0 && l < k) ? B[l + gj * ldb] : 0.0;
+        As[ak + 4 * q][ar] = fa[q];
+        Bs[bk][bc + 16 * q] = fb[q];
       }
       __syncthreads();
-      const int kmax = static_cast<int>(k - l0 < kFK ? k - l0 : kFK);
+      if (l0 + kFK < k) fetch(l0 + kFK);
+      const int kmax = live ? static_cast<int>(k - l0 < kFK ? k - l0 : kFK) : 0;
       for (int kk = 0; kk < kmax; ++kk) {
         double av[4], bv[4];
 #pragma unroll
