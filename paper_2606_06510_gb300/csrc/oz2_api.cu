@@ -525,10 +525,12 @@ struct Arrivals {
 // are still arriving: B's scan, flags and magnitude planes run as soon as B
 // is in, and A's scan chunk by chunk as its columns come (the row keys are
 // maxima, merged across chunks).  The results depend on neither.
+// With `private_ws` nobody reads the workspace afterwards, and a short k may
+// take the path that forms no planes and residues (k_short.cu).
 static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B, int64_t ldb,
                       double* C, int64_t ldc, int num_moduli, int quant, int scale, unsigned flags, void* workspace,
                       size_t ws_bytes, void* stream, const ColumnBlocks* blocks, const BlockDone* on_block,
-                      const Arrivals* in = nullptr) {
+                      const Arrivals* in = nullptr, bool private_ws = false) {
   int st = check_sizes(m, n, k, lda, ldb, ldc);
   if (st) return st;
   if (num_moduli < 1 || num_moduli > kMaxModuli) return OZ2_ERR_UNSUPPORTED_R;
@@ -570,6 +572,9 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
   // A skinny C: A's digit planes formed on chip inside the residue GEMM
   // (never stored), only B deconstructed ahead.
   const bool onfly = !simt && !fused && (flags & OZ2_FLAG_ON_THE_FLY) != 0 && modef_applies(m, n, L.k_pad);
+  // A short k: the integer products from base-256 digits, kept where the
+  // digit planes would be.
+  const bool short_k = private_ws && short_k_applies(m, n, k, L.total - L.planes_a);
   int dev = 0;
   cudaGetDevice(&dev);
   HostStats& hs = g_host_stats[dev];
@@ -630,7 +635,10 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
   }
   if (err == cudaSuccess) err = launch_choose_scales(m, n, k, mods, scale, urow, ra, cb, rf, cf, d, e, ds->status, s);
   mark(4);
-  if (err == cudaSuccess)
+  if (short_k) {
+    if (err == cudaSuccess)
+      err = launch_short_digits(m, n, k, A, lda, B, ldb, ra, cb, d, e, rf, cf, pa, s);
+  } else if (err == cudaSuccess)
     err = launch_deconstruct(onfly ? 0 : m, n, k, mods, ds->table_a, ds->table_b, A, lda, B, ldb, d, e, rf, cf, quant,
                              pa, pb, s);
   mark(5);
@@ -642,7 +650,9 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
     const int64_t cols = blocked ? blocks->widths[bi] : n;
     const uint8_t* pb0 = pb + static_cast<size_t>(c0 / kPlaneRows) * (L.k_pad / kPlaneLine) * L.num_planes *
                                   static_cast<size_t>(kPlaneBlock);
-    if (fused) {
+    if (short_k) {
+      err = launch_short_gemm(m, n, k, c0, cols, mods.T, pa, d, e + c0, C + c0 * ldc, ldc, ds->status, s);
+    } else if (fused) {
       err = launch_fused_crt(m, cols, L.k_pad, mods, pa, pb0, d, e + c0, rf, cf + c0, C + c0 * ldc, ldc, res,
                              L.total - L.residues, ds->status, s);
       mark(6);
@@ -851,7 +861,8 @@ int oz2_dgemm(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, con
     cudaGetLastError();
     return OZ2_ERR_ALLOC;
   }
-  st = oz2_dgemm_ex(m, n, k, A, lda, B, ldb, C, ldc, num_moduli, OZ2_QUANT_TZ, OZ2_SCALE_R2, 0, ws, bytes, stream);
+  st = run_stages(m, n, k, A, lda, B, ldb, C, ldc, num_moduli, OZ2_QUANT_TZ, OZ2_SCALE_R2, 0, ws, bytes, stream, nullptr,
+                  nullptr, nullptr, true);
   cudaError_t e2 = cudaFreeAsync(ws, s);
   if (st == OZ2_OK && e2 != cudaSuccess) st = OZ2_ERR_CUDA;
   return st;
@@ -930,7 +941,7 @@ int oz2_dgemm_host(int64_t m, int64_t n, int64_t k, const double* hA, int64_t ld
   if (err == cudaSuccess) {
     if (k > 0) {
       st = run_stages(m, n, k, dA, m, dB, k, dC, m, num_moduli, OZ2_QUANT_TZ, OZ2_SCALE_R2, 0,
-                      buf + bA + bB + bC, ws, stream, &blocks, &copy_back, &in);
+                      buf + bA + bB + bC, ws, stream, &blocks, &copy_back, &in, true);
     } else {  // C = 0
       err = cudaMemsetAsync(dC, 0, sizeof(double) * m * n, s);
       if (err == cudaSuccess) err = copy_back(0, n);

@@ -201,6 +201,11 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// The same without release semantics (see mbar_arrive_remote_relaxed).
+__device__ __forceinline__ void mbar_arrive_relaxed(uint32_t bar) {
+  asm volatile("mbarrier.arrive.relaxed.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -559,6 +564,16 @@ bool modef_applies(int64_t m, int64_t n, int64_t k_pad);
 cudaError_t launch_modef(int64_t m, int64_t n, int64_t k, const Oz2Moduli& mods, const uint32_t* table_a,
                          const double* A, int64_t lda, const int32_t* d, const uint8_t* row_flag, int quant,
                          const uint8_t* planes_b, int16_t* residues, int64_t ldr, Oz2Device* dev, cudaStream_t st);
+// C for k ≤ 64 from base-256 digits of the scaled integers (k_short.cu), no
+// residues: the digits of both operands into `scratch`, then columns
+// [c0, c0 + cols) of C.  T is the range exponent of the scales.
+bool short_k_applies(int64_t m, int64_t n, int64_t k, size_t scratch_bytes);
+cudaError_t launch_short_digits(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
+                                int64_t ldb, const int32_t* ra, const int32_t* cb, const int32_t* d, const int32_t* e,
+                                const uint8_t* row_flag, const uint8_t* col_flag, uint8_t* scratch, cudaStream_t st);
+cudaError_t launch_short_gemm(int64_t m, int64_t n, int64_t k, int64_t c0, int64_t cols, int T, const uint8_t* scratch,
+                              const int32_t* d, const int32_t* e, double* C, int64_t ldc, Oz2Device* dev,
+                              cudaStream_t st);
 cudaError_t launch_native(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda,
                           const double* B, int64_t ldb, double* C, int64_t ldc, cudaStream_t st);
 }  // namespace oz2

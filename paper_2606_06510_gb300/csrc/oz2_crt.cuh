@@ -337,6 +337,69 @@ __device__ __forceinline__ bool crt_value_w128(const int (&c)[R], int E, const O
   return true;
 }
 
+// Nearest double to X·2^E for the signed 160-bit X = T:Mw:L (|X| < 2^159).
+__device__ __forceinline__ double finish_words160(uint32_t T, u64 Mw, u64 L, int E) {
+  // Magnitude of the signed 160-bit X = T:Mw:L.
+  const bool neg = (T >> 31) != 0;
+  if (neg) {
+    L = 0ull - L;
+    const uint32_t c0 = L == 0 ? 1u : 0u;
+    Mw = ~Mw + c0;
+    T = ~T + ((c0 && Mw == 0) ? 1u : 0u);
+  }
+  // Leading 64 bits and a sticky bit for the rest.
+  u64 top64;
+  bool sticky;
+  if (T != 0) {
+    const int z = __clz(T);                      // 0..31
+    const int sh = 32 - z;                       // bits of T
+    top64 = (static_cast<u64>(T) << (64 - sh)) | (Mw >> sh);
+    sticky = (Mw << (64 - sh)) != 0 || L != 0;
+    E += 64 + sh;
+  } else if (Mw != 0) {
+    const int sh = 64 - __clzll(static_cast<long long>(Mw));  // 1..64
+    top64 = sh == 64 ? Mw : (Mw << (64 - sh)) | (L >> sh);
+    sticky = sh == 64 ? L != 0 : (L << (64 - sh)) != 0;
+    E += sh;
+  } else {
+    top64 = L;
+    sticky = false;
+  }
+  return round_to_double(top64, sticky, E, neg);
+}
+
+// The general routine behind finish_signed, out of the way of its registers.
+static __device__ __noinline__ double finish_signed_slow(uint32_t w4, uint32_t w3, uint32_t w2, uint32_t w1, uint32_t w0, int E) {
+  return finish_words160(w4, (static_cast<u64>(w3) << 32) | w2, (static_cast<u64>(w1) << 32) | w0, E);
+}
+
+// Nearest double to X·2^E for the two's complement X = w3:w2:w1:w0, without
+// taking |X| first: the leading 64 bits below the redundant sign bits, read
+// as a signed word, go through the hardware's signed conversion with a sticky
+// bit for the rest in bit 0.  Setting bit 0 of an even word moves a value
+// strictly between it and its successor to the successor, for either sign,
+// and no rounding boundary (a multiple of 2^9) lies between them.
+__device__ __forceinline__ double finish_signed(uint32_t w3, uint32_t w2, uint32_t w1, uint32_t w0, int E) {
+  const uint32_t sg = static_cast<uint32_t>(static_cast<int>(w3) >> 31);
+  const uint32_t y3 = w3 ^ sg, y2 = w2 ^ sg;
+  if ((y3 | y2) == 0 && (w1 ^ sg) >> 31 == 0) {  // a 64-bit integer
+    const long long x = static_cast<long long>((static_cast<u64>(w1) << 32) | w0);
+    if (x == 0) return 0.0;
+    if (E < -1022 || E > 1023 - 64) return finish_signed_slow(sg, w3, w2, w1, w0, E);
+    return __longlong_as_double(__double_as_longlong(__ll2double_rn(x)) + (static_cast<long long>(E) << 52));
+  }
+  const int sh = (y3 ? __clz(y3) : 32 + __clz(y2)) - 1;  // redundant sign bits: 0..63
+  const int ex = E + 64 - sh;                            // X·2^E = (leading word)·2^ex
+  if (ex < -1022 - 62 || ex > 1021 - 62) return finish_signed_slow(sg, w3, w2, w1, w0, E);
+  const bool ge = sh >= 32;
+  const uint32_t x3 = ge ? w2 : w3, x2 = ge ? w1 : w2, x1 = ge ? w0 : w1, x0 = ge ? 0u : w0;
+  const int sp = sh & 31;
+  const uint32_t th = __funnelshift_l(x2, x3, sp), tl = __funnelshift_l(x1, x2, sp);
+  const uint32_t sticky = ((x1 << sp) | x0) != 0 ? 1u : 0u;
+  const long long top = static_cast<long long>((static_cast<u64>(th) << 32) | tl | sticky);  // |top| in [2^62, 2^63]
+  return __longlong_as_double(__double_as_longlong(__ll2double_rn(top)) + (static_cast<long long>(ex) << 52));
+}
+
 // Fast path for r = 14..16 (2^121 < M < 2^148): the same with 160-bit
 // wrap-around sums, since |X| < 2^147.  S' mod 2^160 is formed from word
 // sums over W_k's words 0..3 (below 2^53 for 16 moduli) and word 4's sum
@@ -372,38 +435,12 @@ __device__ __forceinline__ bool crt_value_w160(const int (&c)[R], int E, const O
   const u128 p1 = static_cast<u128>(q) * mods.M[1] + static_cast<u64>(p0 >> 64);
   const u64 pl = static_cast<u64>(p0), pm = static_cast<u64>(p1);
   const uint32_t pt = static_cast<uint32_t>(static_cast<u64>(p1 >> 64) + q * mods.M[2]);
-  u64 L = lo - pl;
+  const u64 L = lo - pl;
   const uint32_t b0 = lo < pl ? 1u : 0u;
-  u64 Mw = mid - pm - b0;
+  const u64 Mw = mid - pm - b0;
   const uint32_t b1 = (mid < pm || (mid == pm && b0)) ? 1u : 0u;
-  uint32_t T = top - pt - b1;
-  // Magnitude of the signed 160-bit X = T:Mw:L.
-  const bool neg = (T >> 31) != 0;
-  if (neg) {
-    L = 0ull - L;
-    const uint32_t c0 = L == 0 ? 1u : 0u;
-    Mw = ~Mw + c0;
-    T = ~T + ((c0 && Mw == 0) ? 1u : 0u);
-  }
-  // Leading 64 bits and a sticky bit for the rest.
-  u64 top64;
-  bool sticky;
-  if (T != 0) {
-    const int z = __clz(T);                      // 0..31
-    const int sh = 32 - z;                       // bits of T
-    top64 = (static_cast<u64>(T) << (64 - sh)) | (Mw >> sh);
-    sticky = (Mw << (64 - sh)) != 0 || L != 0;
-    E += 64 + sh;
-  } else if (Mw != 0) {
-    const int sh = 64 - __clzll(static_cast<long long>(Mw));  // 1..64
-    top64 = sh == 64 ? Mw : (Mw << (64 - sh)) | (L >> sh);
-    sticky = sh == 64 ? L != 0 : (L << (64 - sh)) != 0;
-    E += sh;
-  } else {
-    top64 = L;
-    sticky = false;
-  }
-  out = round_to_double(top64, sticky, E, neg);
+  const uint32_t T = top - pt - b1;
+  out = finish_words160(T, Mw, L, E);
   return true;
 }
 
