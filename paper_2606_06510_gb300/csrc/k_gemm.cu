@@ -220,7 +220,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     __syncwarp();
   } else if (warp == 1) {
     // ---------------- MMA issuer (leader CTA) ----------------
-    if (leader && lane == 0) {
+    if (leader) {  // the whole warp; lane 0 issues
+      const uint32_t me = lane == 0;
       constexpr uint32_t idesc = idesc_f8_f32(kTileM, kTileN);
       // Stage s, operand o, k-chunk kk: the descriptor of stage 0 plus the
       // byte offset >> 4 (the start-address field has room: smem < 256 KiB).
@@ -236,64 +237,58 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         const Unit x = unit_at<MODE>(u, um);
         const int i = x.i;
         const int np = planes_of<MODE>(mods, i);
-        if (!mbar_wait_bounded(acc_empty, accph ^ 1, kWaitLimit)) {
-          ok = false;
-          break;
-        }
+        ok = mbar_wait_warp(acc_empty, accph ^ 1, kWaitLimit);
+        if (!ok) break;
         tc_fence_after();
         for (int64_t kb = x.k_lo; kb < x.k_hi && ok; ++kb) {
           const uint32_t first = kb == x.k_lo ? 0u : 1u;
           if (np == 2) {  // square: stages (d0,e0) and (d1,e1)
             uint32_t s1 = st, p1 = ph;
             next(s1, p1);
-            if (!mbar_wait_bounded(full0 + 8 * st, ph, kWaitLimit) || !mbar_wait_bounded(full0 + 8 * s1, p1, kWaitLimit)) {
-              ok = false;
-              break;
-            }
+            ok = mbar_wait_warp(full0 + 8 * st, ph, kWaitLimit) && mbar_wait_warp(full0 + 8 * s1, p1, kWaitLimit);
+            if (!ok) break;
             tc_fence_after();
             const uint64_t a0 = desc0 + st * (kStageBytes >> 4), b0 = a0 + (kTileBytes >> 4);
             const uint64_t a1 = desc0 + s1 * (kStageBytes >> 4), b1 = a1 + (kTileBytes >> 4);
 #pragma unroll
             for (int kk = 0; kk < kBK / 32; ++kk) {
               const uint32_t acc = kk ? 1u : first;
-              mma_f8_pair(tmem, a0 + 2 * kk, b0 + 2 * kk, idesc, acc);                 // d0·e0
-              mma_f8_pair(tmem + kAccCols, a1 + 2 * kk, b0 + 2 * kk, idesc, acc);      // d1·e0
-              mma_f8_pair(tmem + kAccCols, a0 + 2 * kk, b1 + 2 * kk, idesc, 1u);       // + d0·e1
+              mma_f8_pair(me, tmem, a0 + 2 * kk, b0 + 2 * kk, idesc, acc);                 // d0·e0
+              mma_f8_pair(me, tmem + kAccCols, a1 + 2 * kk, b0 + 2 * kk, idesc, acc);      // d1·e0
+              mma_f8_pair(me, tmem + kAccCols, a0 + 2 * kk, b1 + 2 * kk, idesc, 1u);       // + d0·e1
             }
-            mma_commit_pair_mc(empty0 + 8 * st, 0x3);
-            mma_commit_pair_mc(empty0 + 8 * s1, 0x3);
+            mma_commit_pair_mc(me, empty0 + 8 * st, 0x3);
+            mma_commit_pair_mc(me, empty0 + 8 * s1, 0x3);
             st = s1;
             ph = p1;
             next(st, ph);
           } else {
             for (int p = 0; p < np; ++p) {  // nonsquare: Σ·Σ → acc0; d0e0, -16 d1·e1 → acc1
-              if (!mbar_wait_bounded(full0 + 8 * st, ph, kWaitLimit)) {
-                ok = false;
-                break;
-              }
+              ok = mbar_wait_warp(full0 + 8 * st, ph, kWaitLimit);
+              if (!ok) break;
               tc_fence_after();
               const uint32_t col = p == 0 ? 0u : kAccCols;
               const uint64_t a = desc0 + st * (kStageBytes >> 4), b = a + (kTileBytes >> 4);
 #pragma unroll
               for (int kk = 0; kk < kBK / 32; ++kk) {
                 const uint32_t acc = (kk || p == 2) ? 1u : first;
-                mma_f8_pair(tmem + col, a + 2 * kk, b + 2 * kk, idesc, acc);
+                mma_f8_pair(me, tmem + col, a + 2 * kk, b + 2 * kk, idesc, acc);
               }
-              mma_commit_pair_mc(empty0 + 8 * st, 0x3);
+              mma_commit_pair_mc(me, empty0 + 8 * st, 0x3);
               next(st, ph);
             }
           }
         }
         if (!ok) break;
-        mma_commit_pair_mc(acc_full, 0x3);  // the unit's accumulators complete, both CTAs
+        mma_commit_pair_mc(me, acc_full, 0x3);  // the unit's accumulators complete, both CTAs
         accph ^= 1;
       }
-      if (!ok) {
+      if (!ok && me) {
         ctx.dev->status = kStatusTimeout;
         ctx.dev->timeout_site = 2;
       }
       // All MMAs retired before the tensor memory or the peer's shared memory goes away.
-      mma_commit_pair(drain_bar);
+      mma_commit_pair(me, drain_bar);
       mbar_wait_bounded(drain_bar, 0, kWaitLimit);
     }
     __syncwarp();
@@ -556,17 +551,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     __syncwarp();
   } else if (warp == 1) {
     // ---------------- MMA issuer (leader CTA) ----------------
-    if (leader && lane == 0) {
+    if (leader) {  // the whole warp; lane 0 issues
+      const uint32_t me = lane == 0;
       constexpr uint32_t idesc = idesc_f8_f32(kTileM, kTileN);
       // Stage s, operand o, k-chunk kk: the descriptor of stage 0 plus the
       // byte offset >> 4 (the start-address field has room: smem < 256 KiB).
       const uint64_t desc0 = smem_desc_sw128(smem_u32(smem));
       uint32_t st = 0, ph = 0, accph = 1;  // current stage and its full-barrier parity
-      auto wait_stage = [&]() {
-        if (!mbar_wait_bounded(full0 + 8 * st, ph, kWaitLimit)) ok = false;
-        return ok;
-      };
-      auto release_stage = [&](uint32_t s) { mma_commit_pair_mc(empty0 + 8 * s, 0x3); };
+      auto wait_stage = [&]() { return ok = mbar_wait_warp(full0 + 8 * st, ph, kWaitLimit); };
+      auto release_stage = [&](uint32_t s) { mma_commit_pair_mc(me, empty0 + 8 * s, 0x3); };
       auto next = [&]() {
         if (++st == kStages) {
           st = 0;
@@ -579,7 +572,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         tc_fence_after();
         const uint64_t a = desc0 + st * (kStageBytes >> 4), b = a + (kTileBytes >> 4);
 #pragma unroll
-        for (int kk = 0; kk < kBK / 32; ++kk) mma_f8_pair(tmem + col, a + 2 * kk, b + 2 * kk, idesc, kk ? 1u : acc);
+        for (int kk = 0; kk < kBK / 32; ++kk) mma_f8_pair(me, tmem + col, a + 2 * kk, b + 2 * kk, idesc, kk ? 1u : acc);
         release_stage(st);
         next();
       };
@@ -597,9 +590,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         const uint64_t a1 = desc0 + s1 * (kStageBytes >> 4), b1 = a1 + (kTileBytes >> 4);
 #pragma unroll
         for (int kk = 0; kk < kBK / 32; ++kk) {
-          if (both) mma_f8_pair(tmem, a0 + 2 * kk, b0 + 2 * kk, idesc, kk ? 1u : acc0);
-          mma_f8_pair(tmem + kAccCols, a1 + 2 * kk, b0 + 2 * kk, idesc, kk ? 1u : acc1);
-          mma_f8_pair(tmem + kAccCols, a0 + 2 * kk, b1 + 2 * kk, idesc, 1u);
+          if (both) mma_f8_pair(me, tmem, a0 + 2 * kk, b0 + 2 * kk, idesc, kk ? 1u : acc0);
+          mma_f8_pair(me, tmem + kAccCols, a1 + 2 * kk, b0 + 2 * kk, idesc, kk ? 1u : acc1);
+          mma_f8_pair(me, tmem + kAccCols, a0 + 2 * kk, b1 + 2 * kk, idesc, 1u);
         }
         release_stage(s0);
         release_stage(s1);
@@ -610,14 +603,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         const int slab = residue_slab_steps(square), khi = static_cast<int>(x.k_hi);
         for (int k0 = static_cast<int>(x.k_lo); k0 < khi && ok; k0 += slab) {
           const int k1 = min(k0 + slab, khi), ke = square ? min(k0 + kSplitSteps, k1) : k1;
-          if (!mbar_wait_bounded(acc_empty, accph, kWaitLimit)) ok = false;
+          ok = mbar_wait_warp(acc_empty, accph, kWaitLimit);
           tc_fence_after();
           for (int kb = k0; kb < ke && ok; ++kb) single(0, kb != k0);  // phase A
-          if (ok && !mbar_wait_bounded(acc_empty + 8, accph, kWaitLimit)) ok = false;
+          ok = ok && mbar_wait_warp(acc_empty + 8, accph, kWaitLimit);
           tc_fence_after();
           for (int kb = ke; kb < k1 && ok; ++kb) cross(true, 1u, kb != ke);  // phase M
           if (!ok) break;
-          mma_commit_pair_mc(acc_full, 0x3);  // acc0 complete for this slab, both CTAs
+          mma_commit_pair_mc(me, acc_full, 0x3);  // acc0 complete for this slab, both CTAs
           if (square) {                       // phase B
             for (int kb = k0; kb < ke && ok; ++kb) cross(false, 1u, ke < k1 || kb != k0);
           } else {
@@ -627,16 +620,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
             }
           }
           if (!ok) break;
-          mma_commit_pair_mc(acc_full + 8, 0x3);
+          mma_commit_pair_mc(me, acc_full + 8, 0x3);
           accph ^= 1;
         }
       }
-      if (!ok) {
+      if (!ok && me) {
         ctx.dev->status = kStatusTimeout;
         ctx.dev->timeout_site = 2;
       }
       // All MMAs retired before the tensor memory or the peer's shared memory goes away.
-      mma_commit_pair(drain_bar);
+      mma_commit_pair(me, drain_bar);
       mbar_wait_bounded(drain_bar, 0, kWaitLimit);
     }
     __syncwarp();
@@ -787,15 +780,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kProbeThreads, 1)
   cluster_sync_all();
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
-  if (leader && threadIdx.x == 32) {
+  if (leader && warp == 1) {  // the whole warp; lane 0 issues
+    const uint32_t me = threadIdx.x == 32;
     constexpr uint32_t idesc = idesc_f8_f32(kTileM, kTileN);
     const uint64_t a = smem_desc_sw128(smem_u32(smem)), b = a + (kTileBytes >> 4);
     for (int64_t it = 0; it < iters; ++it) {
       const uint32_t kk = static_cast<uint32_t>(it & 3);
-      mma_f8_pair(tmem, a + 2 * kk, b + 2 * kk, idesc, it ? 1u : 0u);
+      mma_f8_pair(me, tmem, a + 2 * kk, b + 2 * kk, idesc, it ? 1u : 0u);
     }
-    mma_commit_pair(smem_u32(bar));
-    if (!mbar_wait_bounded(smem_u32(bar), 0, kWaitLimit)) {
+    mma_commit_pair(me, smem_u32(bar));
+    if (!mbar_wait_warp(smem_u32(bar), 0, kWaitLimit) && me) {
       dev->status = kStatusTimeout;
       dev->timeout_site = 4;
     }
