@@ -525,8 +525,9 @@ struct Arrivals {
 // are still arriving: B's scan, flags and magnitude planes run as soon as B
 // is in, and A's scan chunk by chunk as its columns come (the row keys are
 // maxima, merged across chunks).  The results depend on neither.
-// With `private_ws` nobody reads the workspace afterwards, and a short k may
-// take the path that forms no planes and residues (k_short.cu).
+// With `private_ws` nobody reads the workspace afterwards, and a short k or a
+// skinny C takes a path that forms no planes and residues (k_short.cu,
+// k_skinny.cu).
 static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B, int64_t ldb,
                       double* C, int64_t ldc, int num_moduli, int quant, int scale, unsigned flags, void* workspace,
                       size_t ws_bytes, void* stream, const ColumnBlocks* blocks, const BlockDone* on_block,
@@ -575,6 +576,11 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
   // A short k: the integer products from base-256 digits, kept where the
   // digit planes would be.
   const bool short_k = private_ws && short_k_applies(m, n, k, L.total - L.planes_a);
+  // Few rows or columns of C: the same, with the tall operand's digits formed
+  // on chip (every column block must qualify).
+  bool skinny = private_ws && !short_k && skinny_applies(m, n, k, L.num_planes, L.total - L.planes_a);
+  for (int b = 0; blocks && b < blocks->count; ++b)
+    skinny = skinny && skinny_applies(m, blocks->widths[b], k, L.num_planes, L.total - L.planes_a);
   int dev = 0;
   cudaGetDevice(&dev);
   HostStats& hs = g_host_stats[dev];
@@ -638,7 +644,7 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
   if (short_k) {
     if (err == cudaSuccess)
       err = launch_short_digits(m, n, k, A, lda, B, ldb, ra, cb, d, e, rf, cf, pa, s);
-  } else if (err == cudaSuccess)
+  } else if (!skinny && err == cudaSuccess)
     err = launch_deconstruct(onfly ? 0 : m, n, k, mods, ds->table_a, ds->table_b, A, lda, B, ldb, d, e, rf, cf, quant,
                              pa, pb, s);
   mark(5);
@@ -652,6 +658,9 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
                                   static_cast<size_t>(kPlaneBlock);
     if (short_k) {
       err = launch_short_gemm(m, n, k, c0, cols, mods.T, pa, d, e + c0, C + c0 * ldc, ldc, ds->status, s);
+    } else if (skinny) {
+      err = launch_skinny(m, cols, k, A, lda, B + c0 * ldb, ldb, ra, cb + c0, d, e + c0, rf, cf + c0, pa, C + c0 * ldc,
+                          ldc, ds->status, s);
     } else if (fused) {
       err = launch_fused_crt(m, cols, L.k_pad, mods, pa, pb0, d, e + c0, rf, cf + c0, C + c0 * ldc, ldc, res,
                              L.total - L.residues, ds->status, s);

@@ -586,6 +586,14 @@ cudaError_t launch_short_digits(int64_t m, int64_t n, int64_t k, const double* A
 cudaError_t launch_short_gemm(int64_t m, int64_t n, int64_t k, int64_t c0, int64_t cols, int T, const uint8_t* scratch,
                               const int32_t* d, const int32_t* e, double* C, int64_t ldc, Oz2Device* dev,
                               cudaStream_t st);
+// C with few rows or columns from base-256 digits formed on chip (k_skinny.cu);
+// `scratch` holds the skinny operand's digits and the parts of the sums;
+// `planes` are the digit planes the residue path would store.
+bool skinny_applies(int64_t m, int64_t n, int64_t k, int planes, size_t scratch_bytes);
+cudaError_t launch_skinny(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B, int64_t ldb,
+                          const int32_t* ra, const int32_t* cb, const int32_t* d, const int32_t* e,
+                          const uint8_t* row_flag, const uint8_t* col_flag, uint8_t* scratch, double* C, int64_t ldc,
+                          Oz2Device* dev, cudaStream_t st);
 cudaError_t launch_native(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda,
                           const double* B, int64_t ldb, double* C, int64_t ldc, cudaStream_t st);
 }  // namespace oz2
