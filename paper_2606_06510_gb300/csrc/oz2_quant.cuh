@@ -49,26 +49,25 @@ __device__ __forceinline__ unsigned long long quantise_abs(const Split& s, int d
 }
 
 // Truncating quantisation (Eq. scale, TZ): Ã = trunc(x·2^d) as a 64-bit two's
-// complement word, for rows with d ≤ kTzFastMaxD.  With x = ±M·2^(sh - d), M < 2^53, Ã = ±⌊M·2^10 / 2^(10 - sh)⌋: the
-// significand is shifted up by 10 (below 2^63) and then right by r = 10 - sh
-// with clamping funnel shifts, so zeros, subnormals and entries that shift
-// out entirely need no branch.  That needs sh ≤ 9: a normal x has M ≥ 2^52
+// complement word, for rows with d ≤ kTzFastMaxD.  With x = ±M·2^(sh - d),
+// M < 2^53, Ã = ±⌊M·2^10 / 2^(10 - sh)⌋: the significand is shifted up by 10
+// (below 2^63) and then right by r = 10 - sh with one clamping 64-bit shift, so
+// zeros, subnormals and entries that shift out entirely need no branch.  That needs sh ≤ 9: a normal x has M ≥ 2^52
 // and |Ã| < 2^62, and a subnormal one has sh = d - 1074 ≤ 9 for
 // d ≤ kTzFastMaxD (rows with a larger scale, whose largest entry is itself
 // subnormal, take the general path).  d = -4096 gives Ã = 0 for any x.
 constexpr int kTzFastMaxD = 1083;
 __device__ __forceinline__ unsigned long long quantise_tz(double x, int d) {
   const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
-  const int E = static_cast<int>((hi >> 20) & 0x7FFu);
-  const uint32_t mh = (hi & 0xFFFFFu) | (E ? 0x100000u : 0u);  // M = mh·2^32 + lo
-  const uint32_t r = static_cast<uint32_t>(10 + 1075 - max(E, 1) - d);
-  const uint32_t ph = __funnelshift_l(lo, mh, 10), pl = lo << 10;  // M·2^10
-  const bool wide = r >= 32;
-  const uint32_t x1 = wide ? 0u : ph, x0 = wide ? ph : pl, rr = wide ? r - 32 : r;
-  const uint32_t al = __funnelshift_rc(x0, x1, rr), ah = __funnelshift_rc(x1, 0u, rr);
+  const uint32_t E = (hi >> 20) & 0x7FFu;
+  const uint32_t mh = (min(E, 1u) << 20) + (hi & 0xFFFFFu);  // M = mh·2^32 + lo
+  const uint32_t r = static_cast<uint32_t>(10 + 1075 - d) - max(E, 1u);
+  const unsigned long long m10 = (static_cast<unsigned long long>(__funnelshift_l(lo, mh, 10)) << 32) | (lo << 10);
+  unsigned long long q;
+  asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"(m10), "r"(r));
   const uint32_t sgn = static_cast<uint32_t>(static_cast<int>(hi) >> 31);  // 0 or all ones
-  return ((static_cast<unsigned long long>(ah ^ sgn) << 32) | (al ^ sgn)) -
-                               static_cast<unsigned long long>(static_cast<long long>(static_cast<int>(sgn)));
+  return ((static_cast<unsigned long long>(static_cast<uint32_t>(q >> 32) ^ sgn) << 32) |
+          (static_cast<uint32_t>(q) ^ sgn)) + (sgn & 1u);
 }
 
 // Ã of an entry as a 64-bit two's complement word, any scale and quantiser.
