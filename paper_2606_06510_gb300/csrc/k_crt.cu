@@ -41,13 +41,14 @@ constexpr int crt_min_blocks() {
 // The columns of one thread (two rows, or one at an odd last row): each
 // column's residues are loaded while the previous column is reconstructed,
 // alternating between two buffers.  FAST: both rows present, 4-byte residue
-// loads and 16-byte stores possible; otherwise element-wise accesses.
+// loads possible (and 16-byte stores with `wide_store`); otherwise element-wise
+// accesses.
 // Outputs the fast path leaves go into `fails` as 2·(column iteration) + row
 // (0 or 1), the first kCrtFailSlots of them; returns how many there were.
 template <int R, bool FAST>
 __device__ __forceinline__ int crt_columns(int64_t n, int64_t row, bool pair, int d0, int d1, const Oz2Moduli& mods,
                                            const int16_t* __restrict__ res, int64_t ldr, const int* __restrict__ e,
-                                           double* cbase, int64_t ldc, int (&fails)[kCrtFailSlots]) {
+                                           double* cbase, int64_t ldc, bool wide_store, int (&fails)[kCrtFailSlots]) {
   const int64_t step = gridDim.y;
   const int64_t off_step = step * ldr;
   // Residue matrix k starts at res + k·mstride (the same for every thread,
@@ -81,14 +82,16 @@ __device__ __forceinline__ int crt_columns(int64_t n, int64_t row, bool pair, in
       double val;
       if (!crt_fast<R>(c, -((u ? d1 : d0) + ec), mods, val)) {
         val = __longlong_as_double(kCrtSentinel);
-        if (nfail < kCrtFailSlots) fails[nfail] = 2 * iter + u;
-        ++nfail;
+        if (u == 0 || pair) {
+          if (nfail < kCrtFailSlots) fails[nfail] = 2 * iter + u;
+          ++nfail;
+        }
       }
       v[u] = val;
     }
     ++iter;
     double* out = cbase + col * ldc;
-    if (FAST) {
+    if (FAST && wide_store && pair) {
       *reinterpret_cast<double2*>(out) = make_double2(v[0], v[1]);
     } else {
       out[0] = v[0];
@@ -122,25 +125,24 @@ __device__ __forceinline__ int crt_columns(int64_t n, int64_t row, bool pair, in
   return nfail;
 }
 
-// Rows [row0, row0 + rows) of C.  FAST kernels take row pairs with 4-byte
-// residue loads and 16-byte stores (rows even, residues and C aligned); the
-// other kernel takes any rows element-wise.  The two are separate kernels so
+// FAST kernels take row pairs with 4-byte residue loads and, where C is aligned
+// too (`wide_store`), 16-byte stores; the other kernel takes any residues
+// element-wise.  The two are separate kernels so
 // that each gets its own register allocation.
 template <int R, bool FAST>
 __global__ void __launch_bounds__(kCrtThreads, crt_min_blocks<R, FAST>())
-    crt_kernel(int64_t row0, int64_t rows, int64_t n, const __grid_constant__ Oz2Moduli mods,
+    crt_kernel(int64_t rows, int64_t n, const __grid_constant__ Oz2Moduli mods,
                const int16_t* __restrict__ res, int64_t ldr, const int* __restrict__ d, const int* __restrict__ e,
-               double* __restrict__ C, int64_t ldc) {
+               double* __restrict__ C, int64_t ldc, bool wide_store) {
   pdl_trigger();
   pdl_wait();
-  const int64_t rel = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) * 2;
-  if (rel >= rows) return;
-  const int64_t row = row0 + rel;
-  const bool pair = rel + 1 < rows;
+  const int64_t row = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) * 2;
+  if (row >= rows) return;
+  const bool pair = row + 1 < rows;
   const int d0 = d[row], d1 = pair ? d[row + 1] : 0;
   double* cbase = C + row;
   int fails[kCrtFailSlots];
-  const int nfail = crt_columns<R, FAST>(n, row, pair, d0, d1, mods, res, ldr, e, cbase, ldc, fails);
+  const int nfail = crt_columns<R, FAST>(n, row, pair, d0, d1, mods, res, ldr, e, cbase, ldc, wide_store, fails);
   if (nfail == 0) return;
   // Outputs the fast path left to the exact paths (this thread's own).
   const int64_t step = gridDim.y;
@@ -161,12 +163,12 @@ __global__ void __launch_bounds__(kCrtThreads, crt_min_blocks<R, FAST>())
   }
 }
 
-// One launch over rows [row0, row0 + rows): x covers row pairs, y strides
+// One launch: x covers row pairs, y strides
 // over the columns, about two waves of resident blocks in all.
 template <int R, bool FAST>
-static cudaError_t launch_crt_rows(cudaStream_t st, int64_t row0, int64_t rows, int64_t n, const Oz2Moduli& mods,
+static cudaError_t launch_crt_rows(cudaStream_t st, int64_t rows, int64_t n, const Oz2Moduli& mods,
                                    const int16_t* res, int64_t ldr, const int32_t* d, const int32_t* e, double* C,
-                                   int64_t ldc) {
+                                   int64_t ldc, bool wide_store) {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -178,21 +180,19 @@ static cudaError_t launch_crt_rows(cudaStream_t st, int64_t row0, int64_t rows, 
   gy = gy > 65535 ? 65535 : gy;
   count_launch();
   return launch_dependent(crt_kernel<R, FAST>, dim3(static_cast<unsigned>(gx), static_cast<unsigned>(gy)),
-                          dim3(kCrtThreads), 0, st, row0, rows, n, mods, res, ldr, d, e, C, ldc);
+                          dim3(kCrtThreads), 0, st, rows, n, mods, res, ldr, d, e, C, ldc, wide_store);
 }
 
 template <int R>
 static cudaError_t launch_crt_r(cudaStream_t st, int64_t m, int64_t n, const Oz2Moduli& mods, const int16_t* res,
                                 int64_t ldr, const int32_t* d, const int32_t* e, double* C, int64_t ldc) {
-  const bool vec = (ldr % 2 == 0) && (reinterpret_cast<uintptr_t>(res) % 4 == 0) && (ldc % 2 == 0) &&
-                   (reinterpret_cast<uintptr_t>(C) % 16 == 0);
-  if (!vec) return launch_crt_rows<R, false>(st, 0, m, n, mods, res, ldr, d, e, C, ldc);
-  const int64_t even = m & ~int64_t{1};
-  cudaError_t err = cudaSuccess;
-  if (even > 0) err = launch_crt_rows<R, true>(st, 0, even, n, mods, res, ldr, d, e, C, ldc);
-  if (err == cudaSuccess && even < m)
-    err = launch_crt_rows<R, false>(st, even, 1, n, mods, res, ldr, d, e, C, ldc);
-  return err;
+  // Row pairs need 4-byte aligned residues (an odd last row's partner is then
+  // a pad row of theirs); an odd ldc or an unaligned C, a submatrix, costs the
+  // two results a store each.
+  const bool pairs = (ldr % 2 == 0) && (reinterpret_cast<uintptr_t>(res) % 4 == 0);
+  const bool wide = (ldc % 2 == 0) && (reinterpret_cast<uintptr_t>(C) % 16 == 0);
+  return pairs ? launch_crt_rows<R, true>(st, m, n, mods, res, ldr, d, e, C, ldc, wide)
+               : launch_crt_rows<R, false>(st, m, n, mods, res, ldr, d, e, C, ldc, false);
 }
 
 cudaError_t launch_reconstruct(int64_t m, int64_t n, const Oz2Moduli& mods, const int16_t* residues,

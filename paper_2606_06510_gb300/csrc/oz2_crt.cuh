@@ -221,122 +221,6 @@ __device__ __forceinline__ void mad_word(int c, int lo, int hi, long long& acc64
   acc_hi += static_cast<uint32_t>(c) * static_cast<uint32_t>(hi);
 }
 
-// Nearest double to (-1)^neg·(hi·2^64 + lo)·2^E for hi ≠ 0 (general path).
-__device__ __forceinline__ double round_to_double_big(u64 hi, u64 lo, int E, bool neg) {
-  const int sh = 64 - __clzll(static_cast<long long>(hi));
-  const u64 top = (hi << (64 - sh)) | (lo >> sh);
-  return round_to_double(top, (lo << (64 - sh)) != 0, E + sh, neg);
-}
-
-// Nearest double to X·2^E for X = Hs·2^64 + L (two's complement, |X| < 2^127).
-// The common case (|X| ≥ 2^64, normal result) takes the leading 64 bits with
-// two funnel shifts and lets the hardware conversion round them: a sticky
-// bit for the rest is folded into bit 0, below the rounding position (bit
-// 10), so the conversion's round-to-nearest-even decides as the exact value
-// would.  The exponent is then added to the double's bit pattern.
-__device__ __forceinline__ double finish_words(long long Hs, u64 L, int E) {
-  const bool neg = Hs < 0;
-  u64 hi = static_cast<u64>(Hs), lo = L;
-  if (neg) {
-    lo = 0ull - L;
-    hi = ~hi + (L == 0 ? 1ull : 0ull);
-  }
-  if (hi == 0) return round_to_double(lo, false, E, neg);
-  const uint32_t w3 = static_cast<uint32_t>(hi >> 32), w2 = static_cast<uint32_t>(hi);
-  const uint32_t w1 = static_cast<uint32_t>(lo >> 32), w0 = static_cast<uint32_t>(lo);
-  const int s = w3 ? __clz(w3) : 32 + __clz(w2);  // leading zeros of hi (8..63 for |X| < 2^120)
-  const int e2 = E + 127 - s;                      // exponent of the leading bit of X·2^E
-  if (e2 < -1022 || e2 > 1022) return round_to_double_big(hi, lo, E, neg);
-  const bool ge = s >= 32;
-  const uint32_t x3 = ge ? w2 : w3, x2 = ge ? w1 : w2, x1 = ge ? w0 : w1, x0 = ge ? 0u : w0;
-  const int sp = s & 31;
-  const uint32_t th = __funnelshift_l(x2, x3, sp), tl = __funnelshift_l(x1, x2, sp);
-  const bool sticky = ((x1 << sp) | x0) != 0;
-  const u64 top = (static_cast<u64>(th) << 32) | tl | (sticky ? 1ull : 0ull);  // bit 63 set
-  const long long bits = __double_as_longlong(__ull2double_rn(top)) + (static_cast<long long>(E + 64 - s) << 52);
-  return __longlong_as_double(bits | (neg ? (1ll << 63) : 0ll));
-}
-
-// Fast path for r ≤ 12 (M < 2^112) in 32- and 64-bit words.  With
-// S = Σ_k c_k W_k (≡ X mod M) and W_k/M = y_k/m_k:
-//  * Y = Σ c_k F_k mod 2^64, read as a signed word, is 2^64·X/M up to
-//    Σ|c_k|/2 units, as long as X/M is not within that of ±1/2;
-//  * q = (S - X)/M is the integer nearest to Σ c_k g_k/2^18 - Y/2^64
-//    (evaluated in units of 2^-11): with g_k = round(2^18·y_k/m_k) the
-//    first term is within Σ|c_k|·2^-19 < 2^-6 of S/M, and the sum stays a
-//    32-bit integer for |c_k| < m_k;
-//  * L = X mod 2^64 = Σ c_k (W_k mod 2^64) - q·(M mod 2^64), exactly;
-//  * H = ⌊X/2^64⌋ is the integer nearest to Y·round(M/2^51)/2^77 - L/2^64,
-//    from three 32×32 products (the dropped low product is below 1 unit).
-// For |c_k| < m_k the error of the estimate of X/2^64 is below 2^-3.4, so H
-// is exact.  When |Y| is within about 2^52 of 2^63 (X within M/2^12 of
-// ±M/2, which products bounded by Eq. M-bound never reach) the function
-// returns false and the caller takes Garner's algorithm.
-template <int R>
-__device__ __forceinline__ bool crt_value_w64(const int (&c)[R], int E, const Oz2Moduli& mods, double& out) {
-  long long y0 = 0, l0 = 0;
-  uint32_t y1 = 0, l1 = 0;
-  int g0 = 0;
-#pragma unroll
-  for (int k = 0; k < R; ++k) {
-    mad_word(c[k], mods.crt_fl[k], mods.crt_fh[k], y0, y1);
-    mad_word(c[k], mods.crt_wl[k], mods.crt_wh[k], l0, l1);
-    g0 += c[k] * mods.crt_g[k];
-  }
-  const uint32_t yl = static_cast<uint32_t>(y0);
-  const int yh = static_cast<int>(static_cast<uint32_t>(static_cast<u64>(y0) >> 32) + y1);
-  if ((yh ^ (yh >> 31)) >= 0x7FF00000) return false;
-  const int q = ((g0 >> 7) - (yh >> 21) + 1024) >> 11;
-  l0 -= static_cast<long long>(q) * mods.crt_ml;
-  l1 -= static_cast<uint32_t>(q) * static_cast<uint32_t>(mods.crt_mlh);
-  const u64 L = static_cast<u64>(l0) + (static_cast<u64>(l1) << 32);
-  const long long mid = static_cast<long long>(yh) * mods.crt_m51l +
-                        static_cast<long long>(static_cast<u64>(yl) * static_cast<uint32_t>(mods.crt_m51h));
-  const long long zh = static_cast<long long>(yh) * mods.crt_m51h + (mid >> 32);  // ≈ X/2^51
-  const long long H = (zh - static_cast<long long>(static_cast<uint32_t>(L >> 51)) + 4096) >> 13;
-  out = finish_words(H, L, E);
-  return true;
-}
-
-// Fast path for r = 13 (2^112 < M < 2^121).  |X| < M/2 < 2^120, so X is
-// its own residue mod 2^128 read as a signed 128-bit word, and sums that wrap
-// around mod 2^128 suffice.  With u_k = c_k + coff_k ≥ 0, S = Σ u_k W_k ≡ X
-// (mod M); q = ⌊S/M + 1/2⌋ comes from the 32.32 fixed-point sum
-// Σ u_k F_k + 2^31 as in the five-limb path (returning false when its
-// fraction is within 2^-13 of an integer, X that close to ±M/2); and
-// X = (S − q·M) mod 2^128.  S mod 2^128 is formed from the word sums
-// A_j = Σ u_k w_kj (w_kj the 32-bit words of W_k, j = 0..2; u_k < 2^16.1, so
-// A_j < 2^52) and the top word's sum mod 2^32: four multiply-adds per
-// modulus against the five-limb path's six, and no exact S.
-template <int R>
-__device__ __forceinline__ bool crt_value_w128(const int (&c)[R], int E, const Oz2Moduli& mods, double& out) {
-  u64 a0 = 0, a1 = 0, a2 = 0;
-  uint32_t a3 = 0;
-  u64 Q = 1ull << 31;
-#pragma unroll
-  for (int k = 0; k < R; ++k) {
-    const uint32_t u = static_cast<uint32_t>(c[k] + mods.coff[k]);
-    a0 += static_cast<u64>(u) * mods.crtw[k][0];
-    a1 += static_cast<u64>(u) * mods.crtw[k][1];
-    a2 += static_cast<u64>(u) * mods.crtw[k][2];
-    a3 += u * mods.crtw[k][3];
-    Q += static_cast<u64>(u) * mods.crtf[k];
-  }
-  const uint32_t frac = static_cast<uint32_t>(Q);
-  if (frac < (1u << 19) || frac > 0xFFFFFFFFu - (1u << 19)) return false;
-  const u64 q = Q >> 32;
-  // S mod 2^128 = hi·2^64 + lo.
-  const u64 lo = a0 + (a1 << 32);
-  const u64 hi = (a1 >> 32) + a2 + (static_cast<u64>(a3) << 32) + (lo < a0 ? 1ull : 0ull);
-  // q·M mod 2^128 (q < 2^20).
-  const u64 pl = q * mods.M[0];
-  const u64 ph = q * mods.M[1] + __umul64hi(q, mods.M[0]);
-  const u64 L = lo - pl;
-  const u64 H = hi - ph - (lo < pl ? 1ull : 0ull);
-  out = finish_words(static_cast<long long>(H), L, E);
-  return true;
-}
-
 // Nearest double to X·2^E for the signed 160-bit X = T:Mw:L (|X| < 2^159).
 __device__ __forceinline__ double finish_words160(uint32_t T, u64 Mw, u64 L, int E) {
   // Magnitude of the signed 160-bit X = T:Mw:L.
@@ -400,6 +284,98 @@ __device__ __forceinline__ double finish_signed(uint32_t w3, uint32_t w2, uint32
   return __longlong_as_double(__double_as_longlong(__ll2double_rn(top)) + (static_cast<long long>(ex) << 52));
 }
 
+// The same for the 160-bit X = w4:w3:w2:w1:w0.  Where w4 is more than w3's
+// sign, the upper four words are rounded with the last one as part of the
+// sticky bit (at most 31 redundant sign bits: w1 stays below the leading 64).
+__device__ __forceinline__ double finish_signed160(uint32_t w4, uint32_t w3, uint32_t w2, uint32_t w1, uint32_t w0,
+                                                   int E) {
+  const bool big = static_cast<int>(w4) != static_cast<int>(w3) >> 31;
+  return finish_signed(big ? w4 : w3, big ? w3 : w2, big ? w2 : w1, big ? w1 | (w0 != 0 ? 1u : 0u) : w0,
+                       big ? E + 32 : E);
+}
+
+// Fast path for r ≤ 12 (M < 2^112) in 32- and 64-bit words.  With
+// S = Σ_k c_k W_k (≡ X mod M) and W_k/M = y_k/m_k:
+//  * Y = Σ c_k F_k mod 2^64, read as a signed word, is 2^64·X/M up to
+//    Σ|c_k|/2 units, as long as X/M is not within that of ±1/2;
+//  * q = (S - X)/M is the integer nearest to Σ c_k g_k/2^18 - Y/2^64
+//    (evaluated in units of 2^-11): with g_k = round(2^18·y_k/m_k) the
+//    first term is within Σ|c_k|·2^-19 < 2^-6 of S/M, and the sum stays a
+//    32-bit integer for |c_k| < m_k;
+//  * L = X mod 2^64 = Σ c_k (W_k mod 2^64) - q·(M mod 2^64), exactly;
+//  * H = ⌊X/2^64⌋ is the integer nearest to Y·round(M/2^51)/2^77 - L/2^64,
+//    from three 32×32 products (the dropped low product is below 1 unit).
+// For |c_k| < m_k the error of the estimate of X/2^64 is below 2^-3.4, so H
+// is exact.  When |Y| is within about 2^52 of 2^63 (X within M/2^12 of
+// ±M/2, which products bounded by Eq. M-bound never reach) the function
+// returns false and the caller takes Garner's algorithm.
+template <int R>
+__device__ __forceinline__ bool crt_value_w64(const int (&c)[R], int E, const Oz2Moduli& mods, double& out) {
+  long long y0 = 0, l0 = 0;
+  uint32_t y1 = 0, l1 = 0;
+  int g0 = 0;
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    mad_word(c[k], mods.crt_fl[k], mods.crt_fh[k], y0, y1);
+    mad_word(c[k], mods.crt_wl[k], mods.crt_wh[k], l0, l1);
+    g0 += c[k] * mods.crt_g[k];
+  }
+  const uint32_t yl = static_cast<uint32_t>(y0);
+  const int yh = static_cast<int>(static_cast<uint32_t>(static_cast<u64>(y0) >> 32) + y1);
+  if ((yh ^ (yh >> 31)) >= 0x7FF00000) return false;
+  const int q = ((g0 >> 7) - (yh >> 21) + 1024) >> 11;
+  l0 -= static_cast<long long>(q) * mods.crt_ml;
+  l1 -= static_cast<uint32_t>(q) * static_cast<uint32_t>(mods.crt_mlh);
+  const u64 L = static_cast<u64>(l0) + (static_cast<u64>(l1) << 32);
+  const long long mid = static_cast<long long>(yh) * mods.crt_m51l +
+                        static_cast<long long>(static_cast<u64>(yl) * static_cast<uint32_t>(mods.crt_m51h));
+  const long long zh = static_cast<long long>(yh) * mods.crt_m51h + (mid >> 32);  // ≈ X/2^51
+  const long long H = (zh - static_cast<long long>(static_cast<uint32_t>(L >> 51)) + 4096) >> 13;
+  out = finish_signed(static_cast<uint32_t>(static_cast<u64>(H) >> 32), static_cast<uint32_t>(static_cast<u64>(H)),
+                      static_cast<uint32_t>(L >> 32), static_cast<uint32_t>(L), E);
+  return true;
+}
+
+// Fast path for r = 13 (2^112 < M < 2^121).  |X| < M/2 < 2^120, so X is
+// its own residue mod 2^128 read as a signed 128-bit word, and sums that wrap
+// around mod 2^128 suffice.  With u_k = c_k + coff_k ≥ 0, S = Σ u_k W_k ≡ X
+// (mod M); q = ⌊S/M + 1/2⌋ comes from the 32.32 fixed-point sum
+// Σ u_k F_k + 2^31 as in the five-limb path (returning false when its
+// fraction is within 2^-13 of an integer, X that close to ±M/2); and
+// X = (S − q·M) mod 2^128.  S mod 2^128 is formed from the word sums
+// A_j = Σ u_k w_kj (w_kj the 32-bit words of W_k, j = 0..2; u_k < 2^16.1, so
+// A_j < 2^52) and the top word's sum mod 2^32: four multiply-adds per
+// modulus against the five-limb path's six, and no exact S.
+template <int R>
+__device__ __forceinline__ bool crt_value_w128(const int (&c)[R], int E, const Oz2Moduli& mods, double& out) {
+  u64 a0 = 0, a1 = 0, a2 = 0;
+  uint32_t a3 = 0;
+  u64 Q = 1ull << 31;
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    const uint32_t u = static_cast<uint32_t>(c[k] + mods.coff[k]);
+    a0 += static_cast<u64>(u) * mods.crtw[k][0];
+    a1 += static_cast<u64>(u) * mods.crtw[k][1];
+    a2 += static_cast<u64>(u) * mods.crtw[k][2];
+    a3 += u * mods.crtw[k][3];
+    Q += static_cast<u64>(u) * mods.crtf[k];
+  }
+  const uint32_t frac = static_cast<uint32_t>(Q);
+  if (frac < (1u << 19) || frac > 0xFFFFFFFFu - (1u << 19)) return false;
+  const u64 q = Q >> 32;
+  // S mod 2^128 = hi·2^64 + lo.
+  const u64 lo = a0 + (a1 << 32);
+  const u64 hi = (a1 >> 32) + a2 + (static_cast<u64>(a3) << 32) + (lo < a0 ? 1ull : 0ull);
+  // q·M mod 2^128 (q < 2^20).
+  const u64 pl = q * mods.M[0];
+  const u64 ph = q * mods.M[1] + __umul64hi(q, mods.M[0]);
+  const u64 L = lo - pl;
+  const u64 H = hi - ph - (lo < pl ? 1ull : 0ull);
+  out = finish_signed(static_cast<uint32_t>(H >> 32), static_cast<uint32_t>(H), static_cast<uint32_t>(L >> 32),
+                      static_cast<uint32_t>(L), E);
+  return true;
+}
+
 // Fast path for r = 14..16 (2^121 < M < 2^148): the same with 160-bit
 // wrap-around sums, since |X| < 2^147.  S' mod 2^160 is formed from word
 // sums over W_k's words 0..3 (below 2^53 for 16 moduli) and word 4's sum
@@ -440,7 +416,8 @@ __device__ __forceinline__ bool crt_value_w160(const int (&c)[R], int E, const O
   const u64 Mw = mid - pm - b0;
   const uint32_t b1 = (mid < pm || (mid == pm && b0)) ? 1u : 0u;
   const uint32_t T = top - pt - b1;
-  out = finish_words160(T, Mw, L, E);
+  out = finish_signed160(T, static_cast<uint32_t>(Mw >> 32), static_cast<uint32_t>(Mw), static_cast<uint32_t>(L >> 32),
+                         static_cast<uint32_t>(L), E);
   return true;
 }
 
