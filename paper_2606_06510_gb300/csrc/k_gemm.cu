@@ -454,12 +454,19 @@ __device__ __forceinline__ float unpack_scaled(uint32_t word, int j, float w) {
   return fmaf(w, __uint_as_float(__byte_perm(word, 0x4B40u, j ? 0x5432 : 0x5410)), -w * kPackBias);
 }
 
+// TN: columns of a tile.  256, or 64 for a C so small that its 64-column units
+// fill no more than one wave of the CTA pairs: a unit's time is then the drain
+// of its accumulators, a quarter as long, on four times the pairs.
+template <int TN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     residue_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ Oz2Moduli mods, int64_t k_pad, UnitMap um, EpiCtx ctx) {
+  constexpr int kBTile = TN / 2 * kBK;                 // B rows of a CTA
+  constexpr int kStage = kTileBytes + kBTile;
+  constexpr int kCols = TN / 4;                        // columns of an epilogue warp
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStage);
   // bars: full[S], empty[S], acc_full[2], acc_empty[2], drain
   __shared__ uint32_t tmem_base_s;
 
@@ -486,7 +493,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     prefetch_tensormap(&tmB);
   }
   if (warp == 1) {
-    tmem_alloc_pair(smem_u32(&tmem_base_s), kTmemCols);
+    tmem_alloc_pair(smem_u32(&tmem_base_s), 2 * TN);
     tmem_relinquish_pair();
   }
   tc_fence_before();
@@ -506,8 +513,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
           ok = false;
           return;
         }
-        if (leader) mbar_arrive_expect_tx(full0 + 8 * s, 2u * kStageBytes);
-        const uint32_t sa = smem_u32(smem + s * kStageBytes);
+        if (leader) mbar_arrive_expect_tx(full0 + 8 * s, 2u * kStage);
+        const uint32_t sa = smem_u32(smem + s * kStage);
         tma_load_2d_pair(sa, &tmA, full_leader0 + 8 * s, 0, line_a);
         tma_load_2d_pair(sa + kTileBytes, &tmB, full_leader0 + 8 * s, 0, line_b);
         ++it;
@@ -526,7 +533,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         // of the tensor (zero fill).
         const int pline = mods.plane_off[x.i] * kPlaneRows;
         const int line_a = static_cast<int>((x.tm * 2 + rank) * um.ksteps * kb_lines) + pline;
-        const int line_b = static_cast<int>((x.tn * 2 + rank) * um.ksteps * kb_lines) + pline;
+        const int row_b = static_cast<int>(x.tn) * TN + static_cast<int>(rank) * (TN / 2);
+        const int line_b = static_cast<int>(static_cast<int64_t>(row_b / kPlaneRows) * um.ksteps * kb_lines) + pline +
+                           row_b % kPlaneRows;
         auto blocks = [&](int kb0, int kb1, int p0, int np) {
           for (int kb = kb0; kb < kb1 && ok; ++kb) {
             const int off = kb * kb_lines + p0 * kPlaneRows;
@@ -553,7 +562,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     // ---------------- MMA issuer (leader CTA) ----------------
     if (leader) {  // the whole warp; lane 0 issues
       const uint32_t me = lane == 0;
-      constexpr uint32_t idesc = idesc_f8_f32(kTileM, kTileN);
+      constexpr uint32_t idesc = idesc_f8_f32(kTileM, TN);
       // Stage s, operand o, k-chunk kk: the descriptor of stage 0 plus the
       // byte offset >> 4 (the start-address field has room: smem < 256 KiB).
       const uint64_t desc0 = smem_desc_sw128(smem_u32(smem));
@@ -570,7 +579,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       auto single = [&](uint32_t col, uint32_t acc) {
         if (!wait_stage()) return;
         tc_fence_after();
-        const uint64_t a = desc0 + st * (kStageBytes >> 4), b = a + (kTileBytes >> 4);
+        const uint64_t a = desc0 + st * (kStage >> 4), b = a + (kTileBytes >> 4);
 #pragma unroll
         for (int kk = 0; kk < kBK / 32; ++kk) mma_f8_pair(me, tmem + col, a + 2 * kk, b + 2 * kk, idesc, kk ? 1u : acc);
         release_stage(st);
@@ -586,13 +595,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         const uint32_t s1 = st;
         next();
         tc_fence_after();
-        const uint64_t a0 = desc0 + s0 * (kStageBytes >> 4), b0 = a0 + (kTileBytes >> 4);
-        const uint64_t a1 = desc0 + s1 * (kStageBytes >> 4), b1 = a1 + (kTileBytes >> 4);
+        const uint64_t a0 = desc0 + s0 * (kStage >> 4), b0 = a0 + (kTileBytes >> 4);
+        const uint64_t a1 = desc0 + s1 * (kStage >> 4), b1 = a1 + (kTileBytes >> 4);
 #pragma unroll
         for (int kk = 0; kk < kBK / 32; ++kk) {
           if (both) mma_f8_pair(me, tmem, a0 + 2 * kk, b0 + 2 * kk, idesc, kk ? 1u : acc0);
-          mma_f8_pair(me, tmem + kAccCols, a1 + 2 * kk, b0 + 2 * kk, idesc, kk ? 1u : acc1);
-          mma_f8_pair(me, tmem + kAccCols, a0 + 2 * kk, b1 + 2 * kk, idesc, 1u);
+          mma_f8_pair(me, tmem + TN, a1 + 2 * kk, b0 + 2 * kk, idesc, kk ? 1u : acc1);
+          mma_f8_pair(me, tmem + TN, a0 + 2 * kk, b1 + 2 * kk, idesc, 1u);
         }
         release_stage(s0);
         release_stage(s1);
@@ -615,8 +624,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
             for (int kb = k0; kb < ke && ok; ++kb) cross(false, 1u, ke < k1 || kb != k0);
           } else {
             for (int kb = k0; kb < ke && ok; ++kb) {
-              single(kAccCols, kb != k0);
-              if (ok) single(kAccCols, 1u);
+              single(TN, kb != k0);
+              if (ok) single(TN, 1u);
             }
           }
           if (!ok) break;
@@ -636,19 +645,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   } else {
     // ---------------- epilogue (warps 2..17, both CTAs) ----------------
     const int q = warp & 3;                    // TMEM lane quarter of this warp
-    const int h = (warp - 2) >> 2;             // 64-column quarter of the tile
-    const uint32_t lane_addr = tmem + (static_cast<uint32_t>(32 * q) << 16) + static_cast<uint32_t>(64 * h);
+    const int h = (warp - 2) >> 2;             // column quarter of the tile
+    const uint32_t lane_addr = tmem + (static_cast<uint32_t>(32 * q) << 16) + static_cast<uint32_t>(kCols * h);
     const uint32_t acc_empty_leader = mapa_shared(acc_empty, 0);
     uint32_t accph = 0;
-    uint32_t pk[32];  // this thread's 64 running residues, two to a word
+    uint32_t pk[kCols / 2];  // this thread's running residues, two to a word
     // Columns [c, c + 16) of accumulator a; after the last ones the
     // accumulator is free.  The arrive is relaxed: a release would hold it
     // until the residue stores before it are performed, and the MMAs need no
     // ordering against those.
     auto load16 = [&](int a, int c, uint32_t (&v)[16]) {
-      tmem_ld16(lane_addr + a * kAccCols + c, v);
+      tmem_ld16(lane_addr + a * TN + c, v);
       tmem_ld_wait();
-      if (c == 48) {
+      if (c == kCols - 16) {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_remote_relaxed(acc_empty_leader + 8 * a);
@@ -658,7 +667,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       const Unit x = unit_at<0>(u, um);
       const int i = x.i;
       const int64_t row = x.tm * kTileM + rank * kRows + 32 * q + lane;
-      const int64_t col0 = x.tn * kTileN + 64 * h;
+      const int64_t col0 = x.tn * TN + kCols * h;
       const bool square = mods.sq_base[i] != 0;
       const float mf = static_cast<float>(mods.m[i]);
       const float inv = 1.f / mf;
@@ -681,7 +690,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         }
         tc_fence_after();
 #pragma unroll
-        for (int c = 0; c < 64; c += 16) {
+        for (int c = 0; c < kCols; c += 16) {
           uint32_t v[16];
           load16(0, c, v);
 #pragma unroll
@@ -704,7 +713,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         tc_fence_after();
         const float wp = first ? w0 : 1.f;
 #pragma unroll
-        for (int c = 0; c < 64; c += 16) {
+        for (int c = 0; c < kCols; c += 16) {
           uint32_t v[16];
           load16(1, c, v);
           const int64_t cc = col0 + c;
@@ -742,7 +751,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   tc_fence_before();
   cluster_sync_all();  // neither CTA leaves while the pair's MMAs or loads may touch it
   tc_fence_after();
-  if (warp == 1) tmem_dealloc_pair(tmem, kTmemCols);
+  if (warp == 1) tmem_dealloc_pair(tmem, 2 * TN);
 }
 
 // ---------------------------------------------------------------------------
@@ -1085,7 +1094,7 @@ cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Modu
   um.kparts = 1;
   um.kpart_steps = um.ksteps;
   const size_t smem = gemm_smem_bytes();
-  auto kern = mode == 1 ? plane_gemm_kernel<1> : k_pad == kBK ? plane_gemm_kernel<0> : residue_gemm_kernel;
+  auto kern = mode == 1 ? plane_gemm_kernel<1> : k_pad == kBK ? plane_gemm_kernel<0> : residue_gemm_kernel<kTileN>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (err != cudaSuccess) return err;
   // Persistent grid: as many CTA pairs as can be resident at once.
@@ -1133,6 +1142,18 @@ cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Modu
       err = cudaMemsetAsync(ctx.upart, 0, static_cast<size_t>(m) * ctx.ldu * sizeof(float), st);
       if (err != cudaSuccess) return err;
     }
+  }
+  // A small C in one part: tiles of 64 columns while their units are one wave
+  // (256³: the GEMM stage 15.7 µs in 12 units of 256 columns, 11.8 in 48 of 64).
+  const int64_t ntn64 = (n + 63) / 64;
+  if (mode == 0 && k_pad > kBK && um.kparts == 1 && um.ntm * ntn64 * mods.r <= pairs) {
+    um.ntn = ntn64;
+    um.ntiles = um.ntm * um.ntn;
+    um.nunits = um.ntiles * mods.r;
+    kern = residue_gemm_kernel<64>;  // less shared memory, the same threads: as many pairs fit
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (err != cudaSuccess) return err;
+    if (!make_block_map(&tb, planes_b, n, k_pad, mods.nplanes, 32)) return cudaErrorInvalidValue;
   }
   pairs = std::max<int64_t>(1, std::min<int64_t>(pairs, um.nunits));
   count_launch();

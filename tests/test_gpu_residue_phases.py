@@ -5,7 +5,7 @@ nonsquare modulus one after the other, a square one in three phases whose
 first and last cover the first five k-blocks; the residue then travels from
 K-slab to K-slab in registers.  The sizes sit at the edges of those phases
 (four to seven k-blocks), of the K-slabs (4096 and 32768 k-entries) and of
-the tiles, and the result is compared with the CUDA-core twin, which sums the
+the tiles (of 64 columns where those fill one wave), and the result is compared with the CUDA-core twin, which sums the
 same plane products in sequential k order.
 """
 import pytest
@@ -31,6 +31,8 @@ def oz():
     (1, 1, 129, 16), (130, 260, 256, 8), (257, 17, 512, 16), (300, 255, 640, 8), (256, 256, 641, 8),
     (129, 258, 768, 16), (64, 33, 896, 12), (257, 300, 4096, 8), (40, 272, 4097, 16), (130, 20, 8200, 8),
     (16, 24, 32768, 8), (33, 16, 33409, 8),
+    # 64-column tiles, up to one wave of the CTA pairs, and just past it
+    (256, 384, 200, 12), (256, 385, 200, 12), (130, 65, 300, 16), (100, 127, 4200, 3), (20, 1279, 256, 3),
 ])
 def test_phases_match_the_sequential_twin(oz, m, n, k, r):
     import torch
