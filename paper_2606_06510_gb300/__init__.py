@@ -110,13 +110,18 @@ def _check(code: int, what: str):
         raise Oz2Error(code, what)
 
 
+# (The private getters are what torch.cuda.current_stream() calls; the Stream
+# object it builds around them is 3 µs of a small call.)
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def colmajor(t: torch.Tensor) -> torch.Tensor:
@@ -126,18 +131,20 @@ def colmajor(t: torch.Tensor) -> torch.Tensor:
 
 def _ld(t: torch.Tensor) -> int:
     assert t.dim() == 2, "expected a matrix"
-    if t.numel() == 0:
-        return max(t.shape[0], 1)
-    if t.shape[1] > 1 or t.shape[0] > 1:
-        assert t.stride(0) == 1 or t.shape[0] == 1, "matrices must be column-major (stride(0) == 1)"
-    return max(t.stride(1), t.shape[0], 1)
+    rows, cols = t.shape
+    if rows == 0 or cols == 0:
+        return max(rows, 1)
+    s0, s1 = t.stride()
+    if cols > 1 or rows > 1:
+        assert s0 == 1 or rows == 1, "matrices must be column-major (stride(0) == 1)"
+    return max(s1, rows, 1)
 
 
 def _dev(*ts):
     for t in ts:
         if t is not None:
             assert t.is_cuda, "oz2 operates on CUDA tensors"
-            assert t.is_contiguous() or t.stride(0) == 1 or t.dim() == 1
+            assert t.stride(0) == 1 or t.is_contiguous() or t.dim() == 1
 
 
 # ----------------------------------------------------------------- production
@@ -215,9 +222,8 @@ def oz2_dgemm_ex(A, B, C=None, num_moduli=12, quant="tz", scale="r2", flags=0, w
     assert k == k2
     if C is None:
         C = torch.empty((n, m), dtype=torch.float64, device=A.device).t()
-    size = oz2_workspace_size(m, n, k, num_moduli)
     if workspace is None:
-        workspace = torch.empty(max(size, 1), dtype=torch.uint8, device=A.device)
+        workspace = torch.empty(max(oz2_workspace_size(m, n, k, num_moduli), 1), dtype=torch.uint8, device=A.device)
     _dev(A, B, C)
     _check(lib().oz2_dgemm_ex(m, n, k, _ptr(A), _ld(A), _ptr(B), _ld(B), _ptr(C), _ld(C), num_moduli,
                               QUANT[quant], SCALE[scale], flags, _ptr(workspace), workspace.numel(),

@@ -22,6 +22,7 @@
 // list's length the output is marked with a NaN sentinel and found again by
 // a rescan of the thread's later columns.
 #include "oz2_crt.cuh"
+#include "oz2_gemm.cuh"
 
 namespace oz2 {
 
@@ -169,9 +170,7 @@ template <int R, bool FAST>
 static cudaError_t launch_crt_rows(cudaStream_t st, int64_t rows, int64_t n, const Oz2Moduli& mods,
                                    const int16_t* res, int64_t ldr, const int32_t* d, const int32_t* e, double* C,
                                    int64_t ldc, bool wide_store) {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = num_sms();
   const int64_t gx = ((rows + 1) / 2 + kCrtThreads - 1) / kCrtThreads;
   if (gx > 0x7FFFFFFF) return cudaErrorInvalidValue;
   int64_t gy = (2LL * crt_min_blocks<R, FAST>() * sms + gx - 1) / gx;

@@ -750,8 +750,7 @@ cudaError_t launch_deconstruct(int64_t m, int64_t n, int64_t k, const Oz2Moduli&
   switch (mods.r) {
 #define OZ2_DEC_CASE(R)                                                                                     \
   case R:                                                                                                   \
-    err = cudaFuncSetAttribute(planes_kernel<1, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,            \
-                               static_cast<int>(smem));                                                     \
+    err = allow_smem(reinterpret_cast<const void*>(planes_kernel<1, R>), smem);                             \
     if (err == cudaSuccess)                                                                                 \
       err = launch_dependent(planes_kernel<1, R>, dim3(g0 + g1), dim3(threads), smem, st, va, vb, g0, k, k_pad, 0, \
                              rn, mods);                                                                     \

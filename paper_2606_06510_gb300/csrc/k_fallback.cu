@@ -13,7 +13,7 @@
 // at that rate).
 #include <algorithm>
 
-#include "oz2_common.cuh"
+#include "oz2_gemm.cuh"
 
 namespace oz2 {
 
@@ -129,9 +129,7 @@ __global__ void __launch_bounds__(256) fma_gemm_kernel(int64_t m, int64_t n, int
 }
 
 static int fb_grid() {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = num_sms();
   return sms * 4;
 }
 

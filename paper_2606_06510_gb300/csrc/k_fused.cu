@@ -366,7 +366,7 @@ static cudaError_t launch_fused_r(int64_t m, int64_t n, int64_t k_pad, const Oz2
     return cudaErrorInvalidValue;
   const size_t smem = fused_smem_bytes();
   auto kern = k_pad == kBK ? fused_crt_kernel<true> : fused_crt_kernel<false>;
-  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t err = allow_smem(reinterpret_cast<const void*>(kern), smem);
   if (err != cudaSuccess) return err;
   const int64_t ntiles = ((m + kRows - 1) / kRows) * ((n + kFTileN - 1) / kFTileN);
   const int64_t grid = std::min<int64_t>(num_sms(), ntiles);

@@ -40,6 +40,8 @@
 // GEMM and the magnitude GEMM, whose units are over before such an overlap
 // could start or use one accumulator only.
 #include <algorithm>
+#include <mutex>
+#include <vector>
 
 #include "oz2_gemm.cuh"
 
@@ -1059,6 +1061,84 @@ int64_t magnitude_gemm_kparts(int64_t m, int64_t n, int64_t k_pad, size_t scratc
   return magnitude_kparts(ntiles, k_pad / kBK, pairs, m, n, scratch_bytes);
 }
 
+// ---------------------------------------------------------------------------
+// Device and kernel facts, kept per (kernel, device).  A device's SM count and
+// a kernel's resident clusters on it do not change while a process runs.
+// ---------------------------------------------------------------------------
+namespace {
+struct KernelFact {
+  const void* kernel;
+  int dev;
+  size_t smem;       // dynamic shared memory allowed so far
+  int64_t pairs;     // resident two-CTA clusters (0: not asked yet)
+};
+std::mutex g_fact_mu;
+std::vector<KernelFact> g_facts;
+int g_sms[64];
+
+int current_device() {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return dev;
+}
+KernelFact& fact_of(const void* kernel, int dev) {  // with g_fact_mu held
+  for (KernelFact& f : g_facts)
+    if (f.kernel == kernel && f.dev == dev) return f;
+  g_facts.push_back(KernelFact{kernel, dev, 0, 0});
+  return g_facts.back();
+}
+}  // namespace
+
+int num_sms() {
+  const int dev = current_device();
+  if (dev < 0 || dev >= 64) return 148;
+  std::lock_guard<std::mutex> lk(g_fact_mu);
+  if (!g_sms[dev]) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 148;
+    g_sms[dev] = sms;
+  }
+  return g_sms[dev];
+}
+
+cudaError_t allow_smem(const void* kernel, size_t smem) {
+  const int dev = current_device();
+  std::lock_guard<std::mutex> lk(g_fact_mu);
+  KernelFact& f = fact_of(kernel, dev);
+  if (f.smem >= smem) return cudaSuccess;
+  const cudaError_t err =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (err == cudaSuccess) f.smem = smem;
+  return err;
+}
+
+int64_t resident_pairs(const void* kernel, int threads, size_t smem) {
+  const int64_t most = num_sms() / 2;
+  const int dev = current_device();
+  std::lock_guard<std::mutex> lk(g_fact_mu);
+  KernelFact& f = fact_of(kernel, dev);
+  if (!f.pairs) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(2 * most));
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 2;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess || clusters <= 0) {
+      cudaGetLastError();
+      return most;
+    }
+    f.pairs = std::min<int64_t>(most, clusters);
+  }
+  return f.pairs;
+}
+
 // mode: 0 residues (tensor cores), 1 magnitude (tensor cores),
 //       2 residues (SIMT reference), 3 magnitude (SIMT reference).
 cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Moduli& mods,
@@ -1095,28 +1175,10 @@ cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Modu
   um.kpart_steps = um.ksteps;
   const size_t smem = gemm_smem_bytes();
   auto kern = mode == 1 ? plane_gemm_kernel<1> : k_pad == kBK ? plane_gemm_kernel<0> : residue_gemm_kernel<kTileN>;
-  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t err = allow_smem(reinterpret_cast<const void*>(kern), smem);
   if (err != cudaSuccess) return err;
   // Persistent grid: as many CTA pairs as can be resident at once.
-  int64_t pairs = num_sms() / 2;
-  {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs));
-    cfg.blockDim = dim3(kGemmThreads);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 2;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters > 0)
-      pairs = std::min<int64_t>(pairs, clusters);
-    else
-      cudaGetLastError();
-  }
+  int64_t pairs = resident_pairs(reinterpret_cast<const void*>(kern), kGemmThreads, smem);
   // Split K where the scratch holds the parts (16-byte aligned rows: the
   // fold reads and writes 8 residues at a time).
   if (mode == 0 && partials && reinterpret_cast<uintptr_t>(partials) % 16 == 0 &&
@@ -1135,7 +1197,7 @@ cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Modu
     um.nunits *= um.kparts;
     if (um.kparts > 1) {
       kern = plane_gemm_kernel<1, true>;  // same shared memory and threads, so the same pairs fit
-      err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+      err = allow_smem(reinterpret_cast<const void*>(kern), smem);
       if (err != cudaSuccess) return err;
       ctx.upart = reinterpret_cast<float*>(partials);
       ctx.ldu = magnitude_ldu(n);
@@ -1151,7 +1213,7 @@ cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Modu
     um.ntiles = um.ntm * um.ntn;
     um.nunits = um.ntiles * mods.r;
     kern = residue_gemm_kernel<64>;  // less shared memory, the same threads: as many pairs fit
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    err = allow_smem(reinterpret_cast<const void*>(kern), smem);
     if (err != cudaSuccess) return err;
     if (!make_block_map(&tb, planes_b, n, k_pad, mods.nplanes, 32)) return cudaErrorInvalidValue;
   }
@@ -1182,26 +1244,10 @@ cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Modu
 
 // The rate probe on as many CTA pairs as can be resident at once.
 cudaError_t launch_mma_rate(int64_t iters, Oz2Device* dev, int* pairs_out, cudaStream_t st) {
-  cudaError_t err =
-      cudaFuncSetAttribute(mma_rate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kProbeSmem));
+  const void* kern = reinterpret_cast<const void*>(mma_rate_kernel);
+  const cudaError_t err = allow_smem(kern, kProbeSmem);
   if (err != cudaSuccess) return err;
-  int64_t pairs = num_sms() / 2;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs));
-  cfg.blockDim = dim3(kProbeThreads);
-  cfg.dynamicSmemBytes = kProbeSmem;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = 2;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, mma_rate_kernel, &cfg) == cudaSuccess && clusters > 0)
-    pairs = std::min<int64_t>(pairs, clusters);
-  else
-    cudaGetLastError();
+  const int64_t pairs = resident_pairs(kern, kProbeThreads, kProbeSmem);
   if (pairs_out) *pairs_out = static_cast<int>(pairs);
   count_launch();
   mma_rate_kernel<<<static_cast<unsigned>(2 * pairs), kProbeThreads, kProbeSmem, st>>>(iters, dev);

@@ -505,7 +505,7 @@ cudaError_t launch_short_gemm(int64_t m, int64_t n, int64_t k, int64_t c0, int64
     return cudaErrorInvalidValue;
   auto kern = T > 125 ? short_gemm_kernel<true> : short_gemm_kernel<false>;
   const size_t smem = short_smem();
-  const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t err = allow_smem(reinterpret_cast<const void*>(kern), smem);
   if (err != cudaSuccess) return err;
   count_launch();
   const int64_t grid = std::min<int64_t>(num_sms(), a.nrb * a.nct);

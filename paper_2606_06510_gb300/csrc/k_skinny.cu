@@ -631,7 +631,7 @@ cudaError_t launch_skinny(int64_t m, int64_t n, int64_t k, const double* A, int6
   if (err != cudaSuccess) return err;
   const size_t smem = skinny_smem();
   auto kern = b_tall ? skinny_kernel<true> : skinny_kernel<false>;
-  err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  err = allow_smem(reinterpret_cast<const void*>(kern), smem);
   if (err != cudaSuccess) return err;
   err = launch_dependent(kern, dim3(static_cast<unsigned>(p.grid)), dim3(kSnThreads), smem, st, a);
   if (err != cudaSuccess) return err;

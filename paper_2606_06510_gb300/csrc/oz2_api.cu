@@ -232,6 +232,15 @@ static Oz2Moduli build_moduli(int r, int quant) {
   return c;
 }
 
+// The constants of r moduli, built on first use (they cost some microseconds).
+static const Oz2Moduli& moduli_for(int r, int quant) {
+  static Oz2Moduli table[kMaxModuli + 1][2];
+  static std::once_flag once[kMaxModuli + 1][2];
+  const int q = quant == OZ2_QUANT_RN ? 1 : 0;
+  std::call_once(once[r][q], [&] { table[r][q] = build_moduli(r, quant); });
+  return table[r][q];
+}
+
 // ---------------------------------------------------------------------------
 // Per-device state: the plane table is uploaded once per device.
 // ---------------------------------------------------------------------------
@@ -547,7 +556,7 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
   if (!workspace || ws_bytes < L.total || (reinterpret_cast<uintptr_t>(workspace) & 255)) return OZ2_ERR_ALLOC;
   DeviceState* ds = nullptr;
   if ((st = device_state(&ds)) != OZ2_OK) return st;
-  const Oz2Moduli mods = build_moduli(num_moduli, quant);
+  const Oz2Moduli& mods = moduli_for(num_moduli, quant);
 
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   int32_t* ra = reinterpret_cast<int32_t*>(ws + L.ra);
@@ -1090,7 +1099,7 @@ int oz2_scale(int64_t m, int64_t n, int64_t k, int num_moduli, const double* A, 
   DeviceState* ds = nullptr;
   if ((st = device_state(&ds)) != OZ2_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const Oz2Moduli mods = build_moduli(num_moduli, quant);
+  const Oz2Moduli& mods = moduli_for(num_moduli, quant);
   const int64_t k_pad = (k + kKPad - 1) / kKPad * kKPad;
   count_launch();
   reset_status_kernel<<<1, 1, 0, s>>>(ds->status);
@@ -1115,7 +1124,7 @@ int oz2_deconstruct(int64_t m, int64_t n, int64_t k, int num_moduli, const doubl
   if (k == 0 || !A || !B || !d || !e || !row_flag || !col_flag || !planes_a || !planes_b) return OZ2_ERR_INVALID_ARG;
   DeviceState* ds = nullptr;
   if ((st = device_state(&ds)) != OZ2_OK) return st;
-  const Oz2Moduli mods = build_moduli(num_moduli, quant);
+  const Oz2Moduli& mods = moduli_for(num_moduli, quant);
   return to_status(launch_deconstruct(m, n, k, mods, ds->table_a, ds->table_b, A, lda, B, ldb, d, e, row_flag, col_flag, quant,
                                       planes_a, planes_b, static_cast<cudaStream_t>(stream)));
 }
@@ -1128,7 +1137,7 @@ int oz2_residue_gemm(int64_t m, int64_t n, int64_t k, int num_moduli, const uint
   DeviceState* ds = nullptr;
   int st = device_state(&ds);
   if (st) return st;
-  const Oz2Moduli mods = build_moduli(num_moduli, OZ2_QUANT_TZ);
+  const Oz2Moduli& mods = moduli_for(num_moduli, OZ2_QUANT_TZ);
   const int64_t k_pad = (k + kKPad - 1) / kKPad * kKPad;
   return to_status(launch_plane_gemm(m, n, k_pad, mods, planes_a, planes_b, 0, residues, ldr, nullptr, ds->status,
                                      static_cast<cudaStream_t>(stream)));
@@ -1141,7 +1150,7 @@ int oz2_residue_gemm_simt(int64_t m, int64_t n, int64_t k, int num_moduli, const
   DeviceState* ds = nullptr;
   int st = device_state(&ds);
   if (st) return st;
-  const Oz2Moduli mods = build_moduli(num_moduli, OZ2_QUANT_TZ);
+  const Oz2Moduli& mods = moduli_for(num_moduli, OZ2_QUANT_TZ);
   const int64_t k_pad = (k + kKPad - 1) / kKPad * kKPad;
   return to_status(launch_plane_gemm(m, n, k_pad, mods, planes_a, planes_b, 2, residues, ldr, nullptr, ds->status,
                                      static_cast<cudaStream_t>(stream)));
@@ -1152,7 +1161,7 @@ int oz2_reconstruct(int64_t m, int64_t n, int num_moduli, const int16_t* residue
   if (m < 0 || n < 0 || ldr < std::max<int64_t>(1, m) || ldc < std::max<int64_t>(1, m)) return OZ2_ERR_INVALID_ARG;
   if (num_moduli < 1 || num_moduli > kMaxModuli) return OZ2_ERR_UNSUPPORTED_R;
   if (m && n && (!residues || !d || !e || !C)) return OZ2_ERR_INVALID_ARG;
-  const Oz2Moduli mods = build_moduli(num_moduli, OZ2_QUANT_TZ);
+  const Oz2Moduli& mods = moduli_for(num_moduli, OZ2_QUANT_TZ);
   return to_status(
       launch_reconstruct(m, n, mods, residues, ldr, d, e, C, ldc, static_cast<cudaStream_t>(stream)));
 }
