@@ -241,6 +241,8 @@ int oz2_workspace_layout(int64_t m, int64_t n, int64_t k, int num_moduli,
  *                 (exact: integers in units of 2^-2c below 2^24) into an
  *                 m×n buffer in the then unused digit-plane region, and a
  *                 row-maximum kernel follows (one launch more).
+ *                 oz2_dgemm and oz2_dgemm_host, whose launches nobody
+ *                 plans by, make the split only where it is faster.
  * Returns OZ2_OK, OZ2_ERR_INVALID_ARG (null out, negative sizes,
  * cta_pairs < 1) or OZ2_ERR_UNSUPPORTED_R. */
 typedef struct {

@@ -245,7 +245,7 @@ __device__ __forceinline__ void planes_all(std::integer_sequence<int, Is...>, co
 template <int MODE, int R>
 __global__ void __launch_bounds__(TileShape<MODE>::kThreads, TileShape<MODE>::kBlocksPerSm) planes_kernel(OperandView X0, OperandView X1, int blocks0, int64_t k,
                                                              int64_t k_pad, int clamp_c, int rn,
-                                                             const __grid_constant__ Oz2Moduli mods) {
+                                                             const __grid_constant__ Oz2Moduli mods, float* zero, int64_t zero_count) {
   extern __shared__ __align__(16) uint32_t table[];
   pdl_trigger();
   const bool second = static_cast<int>(blockIdx.x) >= blocks0;
@@ -274,6 +274,11 @@ __global__ void __launch_bounds__(TileShape<MODE>::kThreads, TileShape<MODE>::kB
         if (t0 + j * blockDim.x < words4) reinterpret_cast<uint4*>(table)[t0 + j * blockDim.x] = v[j];
     }
     __syncthreads();
+  }
+  if (MODE == 0) {  // the magnitude GEMM's sums (a multiple of four floats, 16-byte aligned)
+    for (int64_t i = 4 * (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x); i < zero_count;
+         i += 4 * static_cast<int64_t>(gridDim.x) * blockDim.x)
+      *reinterpret_cast<float4*>(zero + i) = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   pdl_wait();  // exponents and flags; the table is constant
 
@@ -703,7 +708,7 @@ cudaError_t launch_magnitude_planes(int64_t m, int64_t n, int64_t k, const doubl
                                     int64_t lda, const double* B, int64_t ldb, const int32_t* ra,
                                     const int32_t* cb, const uint8_t* row_flag,
                                     const uint8_t* col_flag, uint8_t* mag_a, uint8_t* mag_b,
-                                    cudaStream_t st) {
+                                    cudaStream_t st, const MagnitudeSplit* split) {
   const int64_t k_pad = (k + kKPad - 1) / kKPad * kKPad;
   int lk = k <= 1 ? 0 : 64 - __builtin_clzll(static_cast<unsigned long long>(k - 1));
   int c = (24 - lk) / 2;
@@ -717,7 +722,8 @@ cudaError_t launch_magnitude_planes(int64_t m, int64_t n, int64_t k, const doubl
   if (g0 == 0) va = vb;
   count_launch();
   return launch_dependent(planes_kernel<0, 0>, dim3(g0 + g1), dim3(TileShape<0>::kThreads), 0, st, va, vb, g0, k, k_pad,
-                          c, 0, dummy);
+                          c, 0, dummy, split && split->parts > 1 ? split->sums : nullptr,
+                          split && split->parts > 1 ? split->count : int64_t{0});
 }
 
 cudaError_t launch_deconstruct(int64_t m, int64_t n, int64_t k, const Oz2Moduli& mods,
@@ -753,7 +759,7 @@ cudaError_t launch_deconstruct(int64_t m, int64_t n, int64_t k, const Oz2Moduli&
     err = allow_smem(reinterpret_cast<const void*>(planes_kernel<1, R>), smem);                             \
     if (err == cudaSuccess)                                                                                 \
       err = launch_dependent(planes_kernel<1, R>, dim3(g0 + g1), dim3(threads), smem, st, va, vb, g0, k, k_pad, 0, \
-                             rn, mods);                                                                     \
+                             rn, mods, nullptr, int64_t{0});                                                \
     break;
     OZ2_DEC_CASE(1) OZ2_DEC_CASE(2) OZ2_DEC_CASE(3) OZ2_DEC_CASE(4) OZ2_DEC_CASE(5) OZ2_DEC_CASE(6)
     OZ2_DEC_CASE(7) OZ2_DEC_CASE(8) OZ2_DEC_CASE(9) OZ2_DEC_CASE(10) OZ2_DEC_CASE(11) OZ2_DEC_CASE(12)

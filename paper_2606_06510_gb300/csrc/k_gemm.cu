@@ -1061,6 +1061,27 @@ int64_t magnitude_gemm_kparts(int64_t m, int64_t n, int64_t k_pad, size_t scratc
   return magnitude_kparts(ntiles, k_pad / kBK, pairs, m, n, scratch_bytes);
 }
 
+// A split costs the sums' zeroing, atomics and a launch for the row maxima,
+// about 10 µs; a k-block is 0.27 µs of a tile.  With `only_if_faster` a split
+// that saves fewer than 36 k-blocks is not made (1000×777×1333: 133 µs a call
+// split, 121 unsplit; 1000×1000×8000, 63 k-blocks in 4 parts: 413 and 411;
+// 1024×1024×65536: 2830 and 2916).
+MagnitudeSplit magnitude_split(int64_t m, int64_t n, int64_t k_pad, void* scratch, size_t scratch_bytes,
+                               bool only_if_faster) {
+  MagnitudeSplit sp{1, nullptr, 0};
+  if (!scratch || reinterpret_cast<uintptr_t>(scratch) % 16 != 0) return sp;
+  const void* kern = reinterpret_cast<const void*>(plane_gemm_kernel<1>);
+  if (allow_smem(kern, gemm_smem_bytes()) != cudaSuccess) return sp;
+  const int64_t p =
+      magnitude_gemm_kparts(m, n, k_pad, scratch_bytes, resident_pairs(kern, kGemmThreads, gemm_smem_bytes()));
+  const int64_t ksteps = k_pad / kBK;
+  if (p < 2 || (only_if_faster && ksteps - (ksteps + p - 1) / p < 36)) return sp;
+  sp.parts = p;
+  sp.sums = static_cast<float*>(scratch);
+  sp.count = m * magnitude_ldu(n);
+  return sp;
+}
+
 // ---------------------------------------------------------------------------
 // Device and kernel facts, kept per (kernel, device).  A device's SM count and
 // a kernel's resident clusters on it do not change while a process runs.
@@ -1144,7 +1165,7 @@ int64_t resident_pairs(const void* kernel, int threads, size_t smem) {
 cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Moduli& mods,
                               const uint8_t* planes_a, const uint8_t* planes_b, int mode,
                               int16_t* residues, int64_t ldr, float* urow, Oz2Device* dev, cudaStream_t st,
-                              int16_t* partials, size_t partial_bytes) {
+                              int16_t* partials, size_t partial_bytes, const MagnitudeSplit* split) {
   if (m == 0 || n == 0) return cudaSuccess;
   EpiCtx ctx{residues, urow, dev, m, n, ldr, nullptr, 0};
   if (mode >= 2) {
@@ -1190,20 +1211,16 @@ cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Modu
     if (um.kparts > 1) ctx.res = partials;
   }
   // The magnitude GEMM of a small C with a long k: parts of k, with U's
-  // partial sums in the scratch (`partials`, 16-byte aligned).
-  if (mode == 1 && partials && reinterpret_cast<uintptr_t>(partials) % 16 == 0) {
-    um.kparts = magnitude_kparts(um.ntiles, um.ksteps, pairs, m, n, partial_bytes);
+  // partial sums (zeroed by the caller) in `split`.
+  if (mode == 1 && split && split->parts > 1) {
+    um.kparts = split->parts;
     um.kpart_steps = (um.ksteps + um.kparts - 1) / um.kparts;
     um.nunits *= um.kparts;
-    if (um.kparts > 1) {
-      kern = plane_gemm_kernel<1, true>;  // same shared memory and threads, so the same pairs fit
-      err = allow_smem(reinterpret_cast<const void*>(kern), smem);
-      if (err != cudaSuccess) return err;
-      ctx.upart = reinterpret_cast<float*>(partials);
-      ctx.ldu = magnitude_ldu(n);
-      err = cudaMemsetAsync(ctx.upart, 0, static_cast<size_t>(m) * ctx.ldu * sizeof(float), st);
-      if (err != cudaSuccess) return err;
-    }
+    kern = plane_gemm_kernel<1, true>;  // same shared memory and threads, so the same pairs fit
+    err = allow_smem(reinterpret_cast<const void*>(kern), smem);
+    if (err != cudaSuccess) return err;
+    ctx.upart = split->sums;
+    ctx.ldu = magnitude_ldu(n);
   }
   // A small C in one part: tiles of 64 columns while their units are one wave
   // (256³: the GEMM stage 15.7 µs in 12 units of 256 columns, 11.8 in 48 of 64).

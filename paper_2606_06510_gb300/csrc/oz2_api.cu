@@ -635,14 +635,17 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
   }
   mark(1);
   if (scale == OZ2_SCALE_R2) {
+    // The digit-plane and residue regions are not yet in use: the scratch for
+    // the magnitude GEMM's partial sums when it splits k (as oz2_plan says,
+    // unless nobody asks: then only where that is faster).
+    const MagnitudeSplit split = simt ? MagnitudeSplit{1, nullptr, 0}
+                                      : magnitude_split(m, n, L.k_pad, pa, L.total - L.planes_a, private_ws);
     if (err == cudaSuccess)
-      err = launch_magnitude_planes(m, in ? 0 : n, k, A, lda, B, ldb, ra, cb, rf, cf, mag_a, mag_b, s);
+      err = launch_magnitude_planes(m, in ? 0 : n, k, A, lda, B, ldb, ra, cb, rf, cf, mag_a, mag_b, s, &split);
     mark(2);
-    // The digit-plane and residue regions are not yet in use: the scratch
-    // for the magnitude GEMM's partial sums when it splits k.
     if (err == cudaSuccess)
-      err = launch_plane_gemm(m, n, L.k_pad, mods, mag_a, mag_b, simt ? 3 : 1, nullptr, 0, urow, ds->status, s,
-                              reinterpret_cast<int16_t*>(pa), L.total - L.planes_a);
+      err = launch_plane_gemm(m, n, L.k_pad, mods, mag_a, mag_b, simt ? 3 : 1, nullptr, 0, urow, ds->status, s, nullptr, 0,
+                              &split);
     mark(3);
   } else {
     mark(2);

@@ -515,11 +515,21 @@ struct ScanOut {
 cudaError_t launch_scan(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda,
                         const double* B, int64_t ldb, unsigned flags, ScanOut out,
                         Oz2Device* dev, cudaStream_t st, bool zero_keys);
+// The magnitude GEMM's split along k: its parts (1: none) and the m×n FP32 sums
+// they add into, `count` floats, which must be zero before it runs.
+struct MagnitudeSplit {
+  int64_t parts;
+  float* sums;
+  int64_t count;
+};
+MagnitudeSplit magnitude_split(int64_t m, int64_t n, int64_t k_pad, void* scratch, size_t scratch_bytes,
+                               bool only_if_faster);
+// With `split` the sums are zeroed along the way.
 cudaError_t launch_magnitude_planes(int64_t m, int64_t n, int64_t k, const double* A,
                                     int64_t lda, const double* B, int64_t ldb, const int32_t* ra,
                                     const int32_t* cb, const uint8_t* row_flag,
                                     const uint8_t* col_flag, uint8_t* mag_a, uint8_t* mag_b,
-                                    cudaStream_t st);
+                                    cudaStream_t st, const MagnitudeSplit* split = nullptr);
 cudaError_t launch_choose_scales(int64_t m, int64_t n, int64_t k, const Oz2Moduli& mods,
                                  int scale_mode, const float* urow, const int32_t* ra,
                                  const int32_t* cb, const uint8_t* row_flag,
@@ -539,13 +549,13 @@ int64_t residue_gemm_kparts(int64_t m, int64_t n, int64_t k_pad, int r, int nsq,
                             int64_t pairs);
 int64_t magnitude_gemm_kparts(int64_t m, int64_t n, int64_t k_pad, size_t scratch_bytes, int64_t pairs);
 // `partials` (16-byte aligned, `partial_bytes` long, or null) is scratch the
-// residue GEMM may split K into (the parts' residues), and the magnitude GEMM
-// too (the m×n FP32 sums of its parts); it must not overlap the operands,
-// C^(i) or urow.
+// residue GEMM may split K into (the parts' residues); `split` is the magnitude
+// GEMM's.  Neither may overlap the operands, C^(i) or urow.
 cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Moduli& mods,
                               const uint8_t* planes_a, const uint8_t* planes_b, int mode,
                               int16_t* residues, int64_t ldr, float* urow, Oz2Device* dev, cudaStream_t st,
-                              int16_t* partials = nullptr, size_t partial_bytes = 0);
+                              int16_t* partials = nullptr, size_t partial_bytes = 0,
+                              const MagnitudeSplit* split = nullptr);
 // `centred`: every residue lies in [-⌊m_k/2⌋, m_k-1-⌊m_k/2⌋] (as the residue
 // GEMM writes them); otherwise any int16 representative.
 cudaError_t launch_reconstruct(int64_t m, int64_t n, const Oz2Moduli& mods,
