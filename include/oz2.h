@@ -218,8 +218,8 @@ int oz2_workspace_layout(int64_t m, int64_t n, int64_t k, int num_moduli,
  * resident two-CTA clusters) pairs, which is SMs/2 unless another kernel's
  * resources or a partitioned device cut the resident clusters; the plan
  * matches a call only for the pair count that call used.
- *   kparts        parts of k per residue-GEMM unit in oz2_dgemm_ex and
- *                 oz2_dgemm (1: no split).  A small C with a long k fills
+ *   kparts        parts of k per residue-GEMM unit in oz2_dgemm_ex (1: no split;
+ *                 oz2_dgemm may take other parts, for the same result).  A small C with a long k fills
  *                 few waves of the CTA pairs; each unit then covers 1/kparts
  *                 of the k-blocks, and a fold sums the parts' residues mod m.
  *   host_blocks   column blocks of oz2_dgemm_host (1 to 8).  The blocks run

@@ -1015,6 +1015,31 @@ int64_t residue_gemm_kparts(int64_t m, int64_t n, int64_t k_pad, int r, int nsq,
   return choose_kparts(ntiles, r, nsq, k_pad / kBK, pairs, m, n, max_parts);
 }
 
+// The parts oz2_dgemm takes, whose plan nobody reads: the fastest by an
+// estimate of this kernel, where a unit's time is its k-blocks (0.96 µs each,
+// every modulus alike) and about three more, and the fold moves the partial
+// residues at 5 TB/s; no split for less than a twentieth.  (1024²×65536, r =
+// 12: 192 units of 512 k-blocks in three waves or 960 of 103
+// in thirteen: 2.79 and 2.72 ms a call; 900×800×40000 r = 10 1.42 and 1.38.)
+static int64_t fastest_kparts(int64_t ntiles, int r, int64_t ksteps, int64_t pairs, int64_t m, int64_t n,
+                              int64_t max_parts) {
+  constexpr double kBlock = 0.96, kUnit = 3.0;  // µs per k-block; a unit's overhead in k-blocks
+  int64_t best = 1;
+  double best_cost = 1e300;
+  for (int64_t p = 1; p <= std::max<int64_t>(1, max_parts); ++p) {
+    const int64_t s = (ksteps + p - 1) / p;
+    if (p > 1 && (s < kMinPartSteps || (ksteps + s - 1) / s != p)) continue;
+    const int64_t waves = (ntiles * r * p + pairs - 1) / pairs;
+    double c = static_cast<double>(waves) * (static_cast<double>(s) + kUnit) * kBlock;
+    if (p > 1) c += 3.0 + (static_cast<double>(p) + 1.0) * r * static_cast<double>(m) * static_cast<double>(n) * 2.0 / 5.0e6;
+    if (c < (best == 1 ? 0.95 : 1.0) * best_cost) {
+      best = p;
+      best_cost = c;
+    }
+  }
+  return best;
+}
+
 static size_t gemm_smem_bytes() { return 1024 + static_cast<size_t>(kStages) * kStageBytes + 8 * (2 * kStages + 5); }
 
 // The magnitude GEMM split along k: each part adds its tiles' partial sums
@@ -1165,7 +1190,7 @@ int64_t resident_pairs(const void* kernel, int threads, size_t smem) {
 cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Moduli& mods,
                               const uint8_t* planes_a, const uint8_t* planes_b, int mode,
                               int16_t* residues, int64_t ldr, float* urow, Oz2Device* dev, cudaStream_t st,
-                              int16_t* partials, size_t partial_bytes, const MagnitudeSplit* split) {
+                              int16_t* partials, size_t partial_bytes, const MagnitudeSplit* split, bool fastest) {
   if (m == 0 || n == 0) return cudaSuccess;
   EpiCtx ctx{residues, urow, dev, m, n, ldr, nullptr, 0};
   if (mode >= 2) {
@@ -1206,6 +1231,11 @@ cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Modu
       reinterpret_cast<uintptr_t>(residues) % 16 == 0) {
     const int nheavy_sq = um.nheavy ? um.nsq : mods.r;  // the model's squares
     um.kparts = residue_gemm_kparts(m, n, k_pad, mods.r, nheavy_sq, ldr, partial_bytes, pairs);
+    if (fastest && ldr % 8 == 0) {
+      const size_t part_bytes = static_cast<size_t>(mods.r) * n * ldr * sizeof(int16_t);
+      um.kparts = fastest_kparts(um.ntiles, mods.r, um.ksteps, pairs, m, n,
+                                 std::min<int64_t>(kMaxKParts, static_cast<int64_t>(partial_bytes / part_bytes)));
+    }
     um.kpart_steps = (um.ksteps + um.kparts - 1) / um.kparts;
     um.nunits *= um.kparts;
     if (um.kparts > 1) ctx.res = partials;

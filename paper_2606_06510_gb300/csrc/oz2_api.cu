@@ -685,7 +685,8 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
         // The magnitude planes are dead once the scales are chosen: their
         // region is the scratch for the partial residues of a split-K GEMM.
         err = launch_plane_gemm(m, cols, L.k_pad, mods, pa, pb0, simt ? 2 : 0, res, L.res_ld, nullptr, ds->status, s,
-                                reinterpret_cast<int16_t*>(mag_a), L.planes_a - L.mag_a);
+                                reinterpret_cast<int16_t*>(mag_a), L.planes_a - L.mag_a, nullptr,
+                                private_ws && !blocked);
       }
       mark(6);
       if (err == cudaSuccess)

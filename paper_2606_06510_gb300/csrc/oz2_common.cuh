@@ -550,12 +550,13 @@ int64_t residue_gemm_kparts(int64_t m, int64_t n, int64_t k_pad, int r, int nsq,
 int64_t magnitude_gemm_kparts(int64_t m, int64_t n, int64_t k_pad, size_t scratch_bytes, int64_t pairs);
 // `partials` (16-byte aligned, `partial_bytes` long, or null) is scratch the
 // residue GEMM may split K into (the parts' residues); `split` is the magnitude
-// GEMM's.  Neither may overlap the operands, C^(i) or urow.
+// GEMM's.  Neither may overlap the operands, C^(i) or urow.  With `fastest` the
+// parts are not residue_gemm_kparts' but this library's own best estimate.
 cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Moduli& mods,
                               const uint8_t* planes_a, const uint8_t* planes_b, int mode,
                               int16_t* residues, int64_t ldr, float* urow, Oz2Device* dev, cudaStream_t st,
                               int16_t* partials = nullptr, size_t partial_bytes = 0,
-                              const MagnitudeSplit* split = nullptr);
+                              const MagnitudeSplit* split = nullptr, bool fastest = false);
 // `centred`: every residue lies in [-⌊m_k/2⌋, m_k-1-⌊m_k/2⌋] (as the residue
 // GEMM writes them); otherwise any int16 representative.
 cudaError_t launch_reconstruct(int64_t m, int64_t n, const Oz2Moduli& mods,
