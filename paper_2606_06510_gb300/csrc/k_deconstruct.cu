@@ -243,98 +243,115 @@ __device__ __forceinline__ void planes_all(std::integer_sequence<int, Is...>, co
 // first R moduli (R is a template parameter so the modulus loop unrolls and
 // every per-modulus constant and plane offset is known at compile time).
 template <int MODE, int R>
-__global__ void __launch_bounds__(TileShape<MODE>::kThreads, TileShape<MODE>::kBlocksPerSm) planes_kernel(OperandView X0, OperandView X1, int blocks0, int64_t k,
-                                                             int64_t k_pad, int clamp_c, int rn,
-                                                             const __grid_constant__ Oz2Moduli mods, float* zero, int64_t zero_count) {
+__global__ void __launch_bounds__(TileShape<MODE>::kThreads, TileShape<MODE>::kBlocksPerSm)
+    planes_kernel(OperandView X0, OperandView X1, uint32_t tiles0, uint32_t tiles1, int64_t k, int64_t k_pad, int clamp_c,
+                  int rn, const __grid_constant__ Oz2Moduli mods, float* zero, int64_t zero_count) {
   extern __shared__ __align__(16) uint32_t table[];
   pdl_trigger();
-  const bool second = static_cast<int>(blockIdx.x) >= blocks0;
-  const OperandView X = second ? X1 : X0;
-  const int bid = second ? blockIdx.x - blocks0 : blockIdx.x;
-  const int nblocks = second ? gridDim.x - blocks0 : blocks0;
   using TS = TileShape<MODE>;
-  const int tile_rows = blockDim.x / TS::kThreadsPerRow;
-  const int64_t rows_out = rows_stored<MODE>(X.rows);
-  const int64_t row_tiles = (rows_out + tile_rows - 1) / tile_rows;
-  const int64_t ntiles = row_tiles * (k_pad / TS::kSeg);
+  const uint32_t tile_rows = blockDim.x / TS::kThreadsPerRow;
   const int part = threadIdx.x & (TS::kThreadsPerRow - 1);
   const int rloc = threadIdx.x / TS::kThreadsPerRow;
-  if (MODE == 1) {
-    // The block's copy of the table, 16 bytes a load and four loads in flight
-    // (word by word the copy alone took 6 µs of a one-tile block's time).
-    const uint4* src = reinterpret_cast<const uint4*>(X.table);
-    const int words4 = (mods.table_entries + 3) >> 2;
-    for (int t0 = threadIdx.x; t0 < words4; t0 += 4 * blockDim.x) {
-      uint4 v[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (t0 + j * blockDim.x < words4) v[j] = __ldg(src + t0 + j * blockDim.x);
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (t0 + j * blockDim.x < words4) reinterpret_cast<uint4*>(table)[t0 + j * blockDim.x] = v[j];
-    }
-    __syncthreads();
-  }
   if (MODE == 0) {  // the magnitude GEMM's sums (a multiple of four floats, 16-byte aligned)
     for (int64_t i = 4 * (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x); i < zero_count;
          i += 4 * static_cast<int64_t>(gridDim.x) * blockDim.x)
       *reinterpret_cast<float4*>(zero + i) = make_float4(0.f, 0.f, 0.f, 0.f);
+    pdl_wait();  // exponents and flags
   }
-  pdl_wait();  // exponents and flags; the table is constant
-
-  for (int64_t tile = bid; tile < ntiles; tile += nblocks) {
-    const int64_t kt = tile / row_tiles;  // consecutive blocks share a k-slice of many rows
-    const int64_t row = (tile - kt * row_tiles) * tile_rows + rloc;
-    if (row >= rows_out) continue;
-    const int64_t l0 = kt * TS::kSeg + part * kElems;
-    const bool pad = row >= X.rows;  // pad rows of the last block: zero digits
-    double x[kElems];
-    if (pad) {
-#pragma unroll
-      for (int e = 0; e < kElems; ++e) x[e] = 0.0;
-    } else {
-      load8(X, row, l0, k, x);  // entries of rows zeroed by the flags are replaced below
+  // Every block walks A's tiles and then B's, gridDim.x apart, so that all end
+  // within a tile of each other (with blocks of their own the operands did not:
+  // a tenth of the time some SMs had none left).
+  uint32_t tile = blockIdx.x;
+#pragma unroll 1
+  for (int op = 0; op < 2; ++op) {
+    const OperandView X = op ? X1 : X0;
+    const uint32_t ntiles = op ? tiles1 : tiles0;
+    if (tile >= ntiles) {
+      tile -= ntiles;
+      continue;
     }
-    const bool zero_row = pad || (X.flag[row] & 2) != 0;
-    const int ex = pad ? 0 : X.exps[row];
-    // Magnitude plane: row-major rows × k_pad.  Digit planes: 128 × 128-byte
-    // blocks, those of one (row block, k-block) consecutive.
-    uint8_t* dst =
-        MODE == 0 ? X.out + static_cast<size_t>(row) * k_pad + l0
-                  : X.out + ((static_cast<size_t>(row / kPlaneRows) * (k_pad / kPlaneLine) + l0 / kPlaneLine) *
-                                 num_planes(R) * kPlaneBlock +
-                             (row % kPlaneRows) * kPlaneLine + l0 % kPlaneLine);
-    const bool fast_tz = MODE == 1 && !rn && ex <= kTzFastMaxD;
-    if (zero_row && !fast_tz) {  // the fast truncating path zeroes through its scale
+    if (MODE == 1) {
+      // The block's copy of the operand's table, 16 bytes a load and four loads
+      // in flight (word by word the copy alone took 6 µs of a one-tile block's
+      // time).
+      const uint4* src = reinterpret_cast<const uint4*>(X.table);
+      const int words4 = (mods.table_entries + 3) >> 2;
+      __syncthreads();  // the other operand's is no longer read
+      for (int t0 = threadIdx.x; t0 < words4; t0 += 4 * blockDim.x) {
+        uint4 v[4];
 #pragma unroll
-      for (int e = 0; e < kElems; ++e) x[e] = 0.0;
-    }
-
-    if (MODE == 0) {
-      uint32_t code[kElems];
+        for (int j = 0; j < 4; ++j)
+          if (t0 + j * blockDim.x < words4) v[j] = __ldg(src + t0 + j * blockDim.x);
 #pragma unroll
-      for (int e = 0; e < kElems; ++e) code[e] = magnitude_code(x[e], ex, clamp_c);
-      *reinterpret_cast<uint2*>(dst) = make_uint2(code[0] | (code[1] << 8) | (code[2] << 16) | (code[3] << 24),
-                                                  code[4] | (code[5] << 8) | (code[6] << 16) | (code[7] << 24));
-    } else {
-      // Quantise (Eq. scale) and split Ã, a 64-bit two's complement word,
-      // into 21-bit limbs.
-      Limbs L;
-      if (fast_tz) {
-        const int d = zero_row ? -4096 : ex;
-#pragma unroll
-        for (int e = 0; e < kElems; ++e) quantise_tz_limbs(x[e], d, L, e);
-      } else {
-#pragma unroll
-        for (int e = 0; e < kElems; ++e) {
-          const Split sp = split_double(x[e]);
-          const unsigned long long a = quantise_abs(sp, ex, rn != 0);
-          const unsigned long long t = sp.neg ? 0ull - a : a;
-          set_limbs(L, e, static_cast<uint32_t>(t), static_cast<int>(t >> 32));
-        }
+        for (int j = 0; j < 4; ++j)
+          if (t0 + j * blockDim.x < words4) reinterpret_cast<uint4*>(table)[t0 + j * blockDim.x] = v[j];
       }
-      planes_all(std::make_integer_sequence<int, R>{}, L, table, dst);
+      __syncthreads();
+      pdl_wait();  // exponents and flags; the table is constant
     }
+    const int64_t rows_out = rows_stored<MODE>(X.rows);
+    const uint32_t row_tiles = static_cast<uint32_t>((rows_out + tile_rows - 1) / tile_rows);
+    // Consecutive blocks share a k-slice of many rows.
+    uint32_t kt = tile / row_tiles, rt = tile - kt * row_tiles;
+    const uint32_t dk = gridDim.x / row_tiles, dr = gridDim.x - dk * row_tiles;
+    for (; tile < ntiles; tile += gridDim.x, kt += dk, rt += dr) {
+      if (rt >= row_tiles) {
+        rt -= row_tiles;
+        ++kt;
+      }
+      const int64_t row = static_cast<int64_t>(rt) * tile_rows + rloc;
+      if (row >= rows_out) continue;
+      const int64_t l0 = static_cast<int64_t>(kt) * TS::kSeg + part * kElems;
+      const bool pad = row >= X.rows;  // pad rows of the last block: zero digits
+      double x[kElems];
+      if (pad) {
+#pragma unroll
+        for (int e = 0; e < kElems; ++e) x[e] = 0.0;
+      } else {
+        load8(X, row, l0, k, x);  // entries of rows zeroed by the flags are replaced below
+      }
+      const bool zero_row = pad || (X.flag[row] & 2) != 0;
+      const int ex = pad ? 0 : X.exps[row];
+      // Magnitude plane: row-major rows × k_pad.  Digit planes: 128 × 128-byte
+      // blocks, those of one (row block, k-block) consecutive.
+      uint8_t* dst =
+          MODE == 0 ? X.out + static_cast<size_t>(row) * k_pad + l0
+                    : X.out + ((static_cast<size_t>(row / kPlaneRows) * (k_pad / kPlaneLine) + l0 / kPlaneLine) *
+                                   num_planes(R) * kPlaneBlock +
+                               (row % kPlaneRows) * kPlaneLine + l0 % kPlaneLine);
+      const bool fast_tz = MODE == 1 && !rn && ex <= kTzFastMaxD;
+      if (zero_row && !fast_tz) {  // the fast truncating path zeroes through its scale
+#pragma unroll
+        for (int e = 0; e < kElems; ++e) x[e] = 0.0;
+      }
+
+      if (MODE == 0) {
+        uint32_t code[kElems];
+#pragma unroll
+        for (int e = 0; e < kElems; ++e) code[e] = magnitude_code(x[e], ex, clamp_c);
+        *reinterpret_cast<uint2*>(dst) = make_uint2(code[0] | (code[1] << 8) | (code[2] << 16) | (code[3] << 24),
+                                                    code[4] | (code[5] << 8) | (code[6] << 16) | (code[7] << 24));
+      } else {
+        // Quantise (Eq. scale) and split Ã, a 64-bit two's complement word,
+        // into 21-bit limbs.
+        Limbs L;
+        if (fast_tz) {
+          const int d = zero_row ? -4096 : ex;
+#pragma unroll
+          for (int e = 0; e < kElems; ++e) quantise_tz_limbs(x[e], d, L, e);
+        } else {
+#pragma unroll
+          for (int e = 0; e < kElems; ++e) {
+            const Split sp = split_double(x[e]);
+            const unsigned long long a = quantise_abs(sp, ex, rn != 0);
+            const unsigned long long t = sp.neg ? 0ull - a : a;
+            set_limbs(L, e, static_cast<uint32_t>(t), static_cast<int>(t >> 32));
+          }
+        }
+        planes_all(std::make_integer_sequence<int, R>{}, L, table, dst);
+      }
+    }
+    tile -= ntiles;
   }
 }
 
@@ -689,16 +706,7 @@ static int64_t tiles_of(int64_t rows, int64_t k_pad) {
   return ((rows_stored<MODE>(rows) + TS::kRows - 1) / TS::kRows) * (k_pad / TS::kSeg);
 }
 
-// Split a grid of about `blocks_per_sm` × SMs blocks between the two operands
-// in proportion to their tiles.
-static void split_grid(int64_t t0, int64_t t1, int blocks_per_sm, int* g0, int* g1) {
-  const int64_t cap = static_cast<int64_t>(num_sms()) * blocks_per_sm;
-  const int64_t tot = t0 + t1;
-  int64_t b0 = t0 ? std::max<int64_t>(1, std::min<int64_t>(t0, cap * t0 / std::max<int64_t>(tot, 1))) : 0;
-  int64_t b1 = t1 ? std::max<int64_t>(1, std::min<int64_t>(t1, cap - b0)) : 0;
-  *g0 = static_cast<int>(b0);
-  *g1 = static_cast<int>(b1);
-}
+constexpr int64_t kTilesMax = 0x7FFFFFFF;  // 2^31 tiles are 70 TB of operands
 
 static int vec_ok(const double* base, int64_t row_stride, int64_t k_stride) {
   return k_stride == 1 && (row_stride % 2 == 0) && (reinterpret_cast<uintptr_t>(base) % 16 == 0);
@@ -716,13 +724,13 @@ cudaError_t launch_magnitude_planes(int64_t m, int64_t n, int64_t k, const doubl
   Oz2Moduli dummy{};
   OperandView va{A, 1, lda, m, ra, row_flag, mag_a, nullptr, 0};
   OperandView vb{B, ldb, 1, n, cb, col_flag, mag_b, nullptr, vec_ok(B, ldb, 1)};
-  int g0, g1;
-  split_grid(m ? tiles_of<0>(m, k_pad) : 0, n ? tiles_of<0>(n, k_pad) : 0, TileShape<0>::kBlocksPerSm, &g0, &g1);
-  if (g0 + g1 == 0) return cudaSuccess;
-  if (g0 == 0) va = vb;
+  const int64_t t0 = m ? tiles_of<0>(m, k_pad) : 0, t1 = n ? tiles_of<0>(n, k_pad) : 0;
+  if (t0 + t1 == 0) return cudaSuccess;
+  if (t0 + t1 > kTilesMax) return cudaErrorInvalidValue;
+  const int64_t grid = std::min<int64_t>(t0 + t1, static_cast<int64_t>(num_sms()) * TileShape<0>::kBlocksPerSm);
   count_launch();
-  return launch_dependent(planes_kernel<0, 0>, dim3(g0 + g1), dim3(TileShape<0>::kThreads), 0, st, va, vb, g0, k, k_pad,
-                          c, 0, dummy, split && split->parts > 1 ? split->sums : nullptr,
+  return launch_dependent(planes_kernel<0, 0>, dim3(static_cast<unsigned>(grid)), dim3(TileShape<0>::kThreads), 0, st, va,
+                          vb, t0, t1, k, k_pad, c, 0, dummy, split && split->parts > 1 ? split->sums : nullptr,
                           split && split->parts > 1 ? split->count : int64_t{0});
 }
 
@@ -747,10 +755,9 @@ cudaError_t launch_deconstruct(int64_t m, int64_t n, int64_t k, const Oz2Moduli&
     t0 *= 4;
     t1 *= 4;
   }
-  int g0, g1;
-  split_grid(t0, t1, per_sm, &g0, &g1);
-  if (g0 + g1 == 0) return cudaSuccess;
-  if (g0 == 0) va = vb;
+  if (t0 + t1 == 0) return cudaSuccess;
+  if (t0 + t1 > kTilesMax) return cudaErrorInvalidValue;
+  const unsigned grid = static_cast<unsigned>(std::min<int64_t>(t0 + t1, static_cast<int64_t>(num_sms()) * per_sm));
   cudaError_t err = cudaSuccess;
   count_launch();
   switch (mods.r) {
@@ -758,7 +765,7 @@ cudaError_t launch_deconstruct(int64_t m, int64_t n, int64_t k, const Oz2Moduli&
   case R:                                                                                                   \
     err = allow_smem(reinterpret_cast<const void*>(planes_kernel<1, R>), smem);                             \
     if (err == cudaSuccess)                                                                                 \
-      err = launch_dependent(planes_kernel<1, R>, dim3(g0 + g1), dim3(threads), smem, st, va, vb, g0, k, k_pad, 0, \
+      err = launch_dependent(planes_kernel<1, R>, dim3(grid), dim3(threads), smem, st, va, vb, t0, t1, k, k_pad, 0, \
                              rn, mods, nullptr, int64_t{0});                                                \
     break;
     OZ2_DEC_CASE(1) OZ2_DEC_CASE(2) OZ2_DEC_CASE(3) OZ2_DEC_CASE(4) OZ2_DEC_CASE(5) OZ2_DEC_CASE(6)
