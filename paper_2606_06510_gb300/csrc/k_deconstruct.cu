@@ -256,8 +256,31 @@ __global__ void __launch_bounds__(TileShape<MODE>::kThreads, TileShape<MODE>::kB
     for (int64_t i = 4 * (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x); i < zero_count;
          i += 4 * static_cast<int64_t>(gridDim.x) * blockDim.x)
       *reinterpret_cast<float4*>(zero + i) = make_float4(0.f, 0.f, 0.f, 0.f);
-    pdl_wait();  // exponents and flags
   }
+  const int words4 = (mods.table_entries + 3) >> 2;  // 16-byte words of a table
+  if (MODE == 1) {
+    // The block's copies of the tables of the operands it has tiles of, 16 bytes
+    // a load and four loads in flight (word by word one copy took 6 µs of a
+    // one-tile block's time).
+    const uint32_t to_b = tiles0 > blockIdx.x ? (tiles0 - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+#pragma unroll 1
+    for (int op = 0; op < 2; ++op) {
+      if (op ? blockIdx.x + to_b * gridDim.x >= tiles0 + tiles1 : blockIdx.x >= tiles0) continue;
+      const uint4* src = reinterpret_cast<const uint4*>(op ? X1.table : X0.table);
+      uint4* dst = reinterpret_cast<uint4*>(table) + op * words4;
+      for (int t0 = threadIdx.x; t0 < words4; t0 += 4 * blockDim.x) {
+        uint4 v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (t0 + j * blockDim.x < words4) v[j] = __ldg(src + t0 + j * blockDim.x);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (t0 + j * blockDim.x < words4) dst[t0 + j * blockDim.x] = v[j];
+      }
+    }
+    __syncthreads();
+  }
+  pdl_wait();  // exponents and flags; the tables are constant
   // Every block walks A's tiles and then B's, gridDim.x apart, so that all end
   // within a tile of each other (with blocks of their own the operands did not:
   // a tenth of the time some SMs had none left).
@@ -269,25 +292,6 @@ __global__ void __launch_bounds__(TileShape<MODE>::kThreads, TileShape<MODE>::kB
     if (tile >= ntiles) {
       tile -= ntiles;
       continue;
-    }
-    if (MODE == 1) {
-      // The block's copy of the operand's table, 16 bytes a load and four loads
-      // in flight (word by word the copy alone took 6 µs of a one-tile block's
-      // time).
-      const uint4* src = reinterpret_cast<const uint4*>(X.table);
-      const int words4 = (mods.table_entries + 3) >> 2;
-      __syncthreads();  // the other operand's is no longer read
-      for (int t0 = threadIdx.x; t0 < words4; t0 += 4 * blockDim.x) {
-        uint4 v[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (t0 + j * blockDim.x < words4) v[j] = __ldg(src + t0 + j * blockDim.x);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (t0 + j * blockDim.x < words4) reinterpret_cast<uint4*>(table)[t0 + j * blockDim.x] = v[j];
-      }
-      __syncthreads();
-      pdl_wait();  // exponents and flags; the table is constant
     }
     const int64_t rows_out = rows_stored<MODE>(X.rows);
     const uint32_t row_tiles = static_cast<uint32_t>((rows_out + tile_rows - 1) / tile_rows);
@@ -348,7 +352,7 @@ __global__ void __launch_bounds__(TileShape<MODE>::kThreads, TileShape<MODE>::kB
             set_limbs(L, e, static_cast<uint32_t>(t), static_cast<int>(t >> 32));
           }
         }
-        planes_all(std::make_integer_sequence<int, R>{}, L, table, dst);
+        planes_all(std::make_integer_sequence<int, R>{}, L, table + op * 4 * words4, dst);
       }
     }
     tile -= ntiles;
@@ -740,7 +744,7 @@ cudaError_t launch_deconstruct(int64_t m, int64_t n, int64_t k, const Oz2Moduli&
                                const uint8_t* row_flag, const uint8_t* col_flag, int quant,
                                uint8_t* planes_a, uint8_t* planes_b, cudaStream_t st) {
   const int64_t k_pad = (k + kKPad - 1) / kKPad * kKPad;
-  const size_t smem = sizeof(uint32_t) * ((mods.table_entries + 3) & ~3);  // copied in 16-byte words
+  const size_t smem = 2 * sizeof(uint32_t) * ((mods.table_entries + 3) & ~3);  // both tables, in 16-byte words
   const int rn = quant == OZ2_QUANT_RN;
   OperandView va{A, 1, lda, m, d, row_flag, planes_a, table_a, 0};
   OperandView vb{B, ldb, 1, n, e, col_flag, planes_b, table_b, vec_ok(B, ldb, 1)};
