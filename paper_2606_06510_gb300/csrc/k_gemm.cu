@@ -1065,6 +1065,19 @@ __global__ void __launch_bounds__(kRowMaxThreads) plus_one_rowmax_kernel(const f
   }
 }
 
+cudaError_t launch_plus_one_rowmax(const float* U, int64_t m, int64_t n, int64_t ldu, float* urow, Oz2Device* dev,
+                                   cudaStream_t st) {
+  constexpr int64_t rows_per_block = kRowMaxThreads / 32;
+  count_launch();
+  return launch_dependent(plus_one_rowmax_kernel, dim3(static_cast<unsigned>((m + rows_per_block - 1) / rows_per_block)),
+                          dim3(kRowMaxThreads), 0, st, U, m, n, ldu, urow, dev);
+}
+
+// The sums of a magnitude GEMM that adds into U anyway (k_skinny.cu).
+MagnitudeSplit magnitude_sums(int64_t m, int64_t n, void* scratch) {
+  return MagnitudeSplit{2, static_cast<float*>(scratch), m * ((n + 3) / 4 * 4)};
+}
+
 // Parts of k for the magnitude GEMM: its 256×256 tiles fill fewer than half
 // a wave of the CTA pairs only for a small C with a long k; then each tile
 // runs in as many parts as the pairs allow (at most 64, each at least
@@ -1272,12 +1285,7 @@ cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Modu
   // 1024²×65536 2795 and 2873).
   err = launch_dependent(kern, dim3(static_cast<unsigned>(2 * pairs)), dim3(kGemmThreads), smem, st, ta, tb, mods, k_pad,
                          um, ctx);
-  if (err == cudaSuccess && ctx.upart) {
-    count_launch();
-    constexpr int64_t rows_per_block = kRowMaxThreads / 32;
-    err = launch_dependent(plus_one_rowmax_kernel, dim3(static_cast<unsigned>((m + rows_per_block - 1) / rows_per_block)),
-                           dim3(kRowMaxThreads), 0, st, ctx.upart, m, n, ctx.ldu, urow, dev);
-  }
+  if (err == cudaSuccess && ctx.upart) err = launch_plus_one_rowmax(ctx.upart, m, n, ctx.ldu, urow, dev, st);
   if (err == cudaSuccess && mode == 0 && um.kparts > 1) {  // the residue GEMM's parts, folded into C^(i)
     const int64_t row_threads = (m + 7) / 8;
     dim3 g(static_cast<unsigned>((row_threads + kFoldThreads - 1) / kFoldThreads),

@@ -193,6 +193,14 @@ __device__ __forceinline__ long long sn_mad_wide(int a, int b, long long c) {
   asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
   return r;
 }
+__device__ __forceinline__ void mma_f8_by(uint32_t me, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                          uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(me)
+      : "memory");
+}
 // Linear copy of global memory into shared memory, completing on an mbarrier
 // (16-byte aligned, a multiple of 16 bytes).
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
@@ -558,6 +566,222 @@ __global__ void __launch_bounds__(kRows) skinny_finish_kernel(const uint32_t* __
   C[row * tall_stride + col * skinny_stride] = val;
 }
 
+// ---------------------------------------------------------------------------
+// The "+1" pass (§2.4) of a product with few columns: U = ÂB̂ with A's magnitude
+// codes formed on chip, instead of writing their plane and reading it back.  A
+// thread makes the 16 codes of one core-matrix row; the tensor core sums all of
+// a CTA's run of k in FP32 (every partial sum is an integer number of units
+// below 2^24, so their order is free), and the runs add into U, whose row maxima
+// plus_one_rowmax_kernel then takes.  The loads of A bound it: two CTAs an SM
+// (one left a third of them unhidden).  Measured, 16384×16×16384: 0.35 ms for
+// the plane and the GEMM's 0.47 + 0.05 (the call 1.59 → 1.44 ms).
+// ---------------------------------------------------------------------------
+constexpr int kSpK = 64;                               // k-entries of a chunk: two MMA K-steps
+constexpr int kSpATile = kRows * 16;                   // 128 rows × 16 entries
+constexpr int kSpABuf = kSpATile * (kSpK / 16);        // 8 KiB
+constexpr int kSpABufs = 4;
+constexpr int kSpColsMax = 80;                         // columns of the skinny operand, in sixteens
+constexpr int kSpBBuf = kSpColsMax * kSpK;             // 5 KiB
+constexpr int kSpCodeWarps = 16;
+constexpr int kSpThreads = 32 * (kSpCodeWarps + 2);    // MMA issuer, copies of the skinny operand's codes
+
+struct SkinnyPlusArgs {
+  const double* A;
+  int64_t lda, rows, k;
+  int64_t nrb, chunks, total;     // row blocks, chunks of k, their product
+  const int32_t* scan;
+  const uint8_t* flag;
+  int clamp;
+  const uint8_t* codes;           // of B: cols × k_pad bytes
+  int64_t cols, k_pad;
+  int npad;                       // cols to a multiple of 16
+  float* U;                       // row-major, ld = ldu
+  int64_t ldu;
+  Oz2Device* dev;
+};
+
+__global__ void __launch_bounds__(kSpThreads, 2) skinny_plus_one_kernel(const __grid_constant__ SkinnyPlusArgs a) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* sm_a = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sm_b = sm_a + kSpABufs * kSpABuf;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sm_b + kSpABufs * kSpBBuf);
+  __shared__ uint32_t tmem_base_s;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // Codes of both operands ready (16 + 1 warps), a buffer free, a row block's sums ready, drained.
+  const uint32_t full = smem_u32(bars), empty = full + 8 * kSpABufs, accf = empty + 8 * kSpABufs, acce = accf + 8,
+                 drain_bar = acce + 8;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kSpABufs; ++s) {
+      mbar_init(full + 8 * s, kSpCodeWarps + 1);
+      mbar_init(empty + 8 * s, 1);
+    }
+    mbar_init(accf, 1);
+    mbar_init(acce, kSpCodeWarps);
+    mbar_init(drain_bar, 1);
+    fence_barrier_init();
+  }
+  if (warp == kSpCodeWarps) {
+    tmem_alloc(smem_u32(&tmem_base_s), 128);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_base_s;
+  pdl_wait();  // exponents, flags, the skinny operand's codes, U zero
+  const int64_t u0 = a.total * blockIdx.x / gridDim.x, u1 = a.total * (blockIdx.x + 1) / gridDim.x;
+  const int64_t first_rb = u0 / a.chunks;
+  const int64_t first_chunk = u0 - first_rb * a.chunks;
+  const int units = static_cast<int>(u1 - u0);
+  bool ok = true;
+
+  if (warp == kSpCodeWarps + 1) {
+    // ---------------- B's codes ----------------
+    int64_t chunk = first_chunk;
+    for (int t = 0; t < units && ok; ++t) {
+      const uint32_t s = t % kSpABufs;
+      ok = mbar_wait_warp(empty + 8 * s, ((t / kSpABufs) & 1) ^ 1, kWaitLimit);
+      if (!ok) break;
+      uint8_t* dst = sm_b + s * kSpBBuf;
+      const int pieces = a.npad * (kSpK / 16);
+      for (int i = lane; i < pieces; i += 32) {  // 16 codes each: column i / 4, K column i mod 4
+        const int c = i >> 2, kc = i & 3;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (c < a.cols) v = __ldg(reinterpret_cast<const uint4*>(a.codes + c * a.k_pad + chunk * kSpK + 16 * kc));
+        *reinterpret_cast<uint4*>(dst + (kc * a.npad + c) * 16) = v;
+      }
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full + 8 * s);
+      if (++chunk == a.chunks) chunk = 0;
+    }
+    if (!ok && lane == 0) {
+      a.dev->status = kStatusTimeout;
+      a.dev->timeout_site = 17;
+    }
+  } else if (warp == kSpCodeWarps) {
+    // ---------------- MMA issuer ----------------
+    const uint32_t me = lane == 0;
+    const uint32_t idesc = idesc_f8_f32(kRows, a.npad);
+    const uint64_t da = smem_desc_plain(smem_u32(sm_a), kSpATile, 128);
+    const uint64_t db = smem_desc_plain(smem_u32(sm_b), a.npad * 16, 128);
+    int64_t chunk = first_chunk;
+    uint32_t blocks = 0, fresh = 0;  // row blocks begun; whether the sums hold this one's
+    for (int t = 0; t < units && ok; ++t) {
+      const uint32_t s = t % kSpABufs;
+      if (!fresh) ok = mbar_wait_warp(acce, (blocks & 1) ^ 1, kWaitLimit);
+      ok = ok && mbar_wait_warp(full + 8 * s, (t / kSpABufs) & 1, kWaitLimit);
+      if (!ok) break;
+      tc_fence_after();
+#pragma unroll
+      for (int kk = 0; kk < kSpK / 32; ++kk)
+        mma_f8_by(me, tmem, da + s * (kSpABuf >> 4) + kk * (2 * kSpATile >> 4),
+                  db + s * (kSpBBuf >> 4) + kk * (2 * a.npad * 16 >> 4), idesc, kk ? 1u : fresh);
+      sn_commit(me, empty + 8 * s);
+      fresh = 1;
+      if (++chunk == a.chunks || t + 1 == units) {
+        sn_commit(me, accf);
+        chunk = 0;
+        fresh = 0;
+        ++blocks;
+      }
+    }
+    if (!ok && me) {
+      a.dev->status = kStatusTimeout;
+      a.dev->timeout_site = 18;
+    }
+    sn_commit(me, drain_bar);
+    mbar_wait_bounded(drain_bar, 0, kWaitLimit);
+    __syncwarp();
+  } else {
+    // ---------------- A's codes, and the sums ----------------
+    const int rq = warp & 3, cq = warp >> 2;
+    // 16 entries (`part` of a chunk) of a row.
+    const int rloc = 32 * rq + lane, part = cq;
+    const uint32_t lane_addr = tmem + (static_cast<uint32_t>(32 * rq) << 16);
+    int64_t rb = first_rb, chunk = first_chunk;
+    const double* p = nullptr;
+    int ex = 0;
+    bool live = false;
+    auto enter = [&]() {
+      const int64_t row = rb * kRows + rloc;
+      live = row < a.rows && !(a.flag[row] & 2);
+      ex = live ? a.scan[row] : 0;
+      p = a.A + (row < a.rows ? row : a.rows - 1);
+    };
+    auto fetch = [&](int64_t c, double (&x)[16]) {
+      const int64_t l = c * kSpK + part * 16;
+      const double* e = p + l * a.lda;
+      if (l + 16 <= a.k) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j, e += a.lda) x[j] = __ldg(e);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j, e += a.lda) x[j] = l + j < a.k ? __ldg(e) : 0.0;
+      }
+    };
+    enter();
+    double x[16];
+    fetch(chunk, x);
+    uint32_t blocks = 0;
+    for (int t = 0; t < units && ok; ++t) {
+      uint32_t w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        uint32_t v = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v |= magnitude_code(x[4 * j + i], ex, a.clamp) << (8 * i);
+        w[j] = live ? v : 0u;
+      }
+      const bool ends = chunk + 1 == a.chunks || t + 1 == units;
+      const int64_t out_rb = rb;
+      if (t + 1 < units) {
+        if (++chunk == a.chunks) {
+          chunk = 0;
+          ++rb;
+          enter();
+        }
+        fetch(chunk, x);
+      }
+      const uint32_t s = t % kSpABufs;
+      ok = mbar_wait_warp(empty + 8 * s, ((t / kSpABufs) & 1) ^ 1, kWaitLimit);
+      if (!ok) break;
+      *reinterpret_cast<uint4*>(sm_a + s * kSpABuf + part * kSpATile + rloc * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full + 8 * s);
+      if (ends) {  // the row block's sums (of this run) into U
+        ok = mbar_wait_warp(accf, blocks & 1, kWaitLimit);
+        if (!ok) break;
+        tc_fence_after();
+        const int64_t row = out_rb * kRows + 32 * rq + lane;
+        for (int c = 4 * cq; c < a.npad; c += 16) {
+          uint32_t v[4];
+          tmem_ld4(lane_addr + c, v);
+          tmem_ld_wait();
+          if (row < a.rows) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (c + j < a.cols) atomicAdd(a.U + row * a.ldu + c + j, __uint_as_float(v[j]));
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acce);
+        ++blocks;
+      }
+    }
+    if (!ok && lane == 0) {
+      a.dev->status = kStatusTimeout;
+      a.dev->timeout_site = 19;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == kSpCodeWarps) tmem_dealloc(tmem, 128);
+}
+
 static size_t skinny_smem() {
   return 1024 + 2 * static_cast<size_t>(kSnABuf) + kSnBStages * static_cast<size_t>(kSnBChunk) + 8 * (8 + 2 * kSnBStages + 1);
 }
@@ -591,6 +815,43 @@ static SkinnyPlan skinny_plan(int64_t m, int64_t n, int64_t k) {
 // 3.85 against 2.83; 500×64×20000 0.227 against 0.255; 16×16×128 alike.)
 bool skinny_applies(int64_t m, int64_t n, int64_t k, int planes, size_t scratch_bytes) {
   return std::min(m, n) <= kSnCols * ((14 + planes) / 10) && skinny_plan(m, n, k).bytes <= scratch_bytes;
+}
+
+// Where A is larger than L2; below that the plane stays there and the pass only
+// adds a launch (4000×30×4000 alike, 128×48×20000 97 against 126 µs).
+bool skinny_plus_one_applies(int64_t m, int64_t n, int64_t k) { return n <= m && m * k >= (int64_t{1} << 24); }
+
+// U = ÂB̂ into the zeroed sums of `split` (m×n row-major, ld n to a multiple of
+// 4) and its row maxima.  `codes` are B's magnitude codes.
+cudaError_t launch_skinny_plus_one(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const int32_t* ra,
+                                   const uint8_t* row_flag, const uint8_t* codes, const MagnitudeSplit& split,
+                                   float* urow, Oz2Device* dev, cudaStream_t st) {
+  SkinnyPlusArgs a{};
+  a.A = A;
+  a.lda = lda;
+  a.rows = m;
+  a.k = k;
+  a.k_pad = (k + kKPad - 1) / kKPad * kKPad;
+  a.nrb = (m + kRows - 1) / kRows;
+  a.chunks = a.k_pad / kSpK;
+  a.total = a.nrb * a.chunks;
+  a.scan = ra;
+  a.flag = row_flag;
+  a.clamp = magnitude_clamp(k);
+  a.codes = codes;
+  a.cols = n;
+  a.npad = static_cast<int>((n + 15) / 16 * 16);
+  a.U = split.sums;
+  a.ldu = split.count / m;
+  a.dev = dev;
+  const void* kern = reinterpret_cast<const void*>(skinny_plus_one_kernel);
+  const size_t smem = 1024 + kSpABufs * static_cast<size_t>(kSpABuf + kSpBBuf) + 8 * (2 * kSpABufs + 3);
+  cudaError_t err = allow_smem(kern, smem);
+  if (err != cudaSuccess) return err;
+  count_launch();
+  const int64_t grid = std::min<int64_t>(2 * num_sms(), a.total);
+  err = launch_dependent(skinny_plus_one_kernel, dim3(static_cast<unsigned>(grid)), dim3(kSpThreads), smem, st, a);
+  return err != cudaSuccess ? err : launch_plus_one_rowmax(split.sums, m, n, a.ldu, urow, dev, st);
 }
 
 cudaError_t launch_skinny(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B, int64_t ldb,

@@ -634,7 +634,15 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
     err = launch_scan(m, n, k, A, lda, B, ldb, flags, so, ds->status, s, false);
   }
   mark(1);
-  if (scale == OZ2_SCALE_R2) {
+  if (scale == OZ2_SCALE_R2 && skinny && !in && skinny_plus_one_applies(m, n, k)) {
+    // B's codes, U zeroed; then A's on chip.
+    const MagnitudeSplit sums = magnitude_sums(m, n, pa);
+    if (err == cudaSuccess) err = launch_magnitude_planes(0, n, k, A, lda, B, ldb, ra, cb, rf, cf, mag_a, mag_b, s, &sums);
+    mark(2);
+    if (err == cudaSuccess)
+      err = launch_skinny_plus_one(m, n, k, A, lda, ra, rf, mag_b, sums, urow, ds->status, s);
+    mark(3);
+  } else if (scale == OZ2_SCALE_R2) {
     // The digit-plane and residue regions are not yet in use: the scratch for
     // the magnitude GEMM's partial sums when it splits k (as oz2_plan says,
     // unless nobody asks: then only where that is faster).

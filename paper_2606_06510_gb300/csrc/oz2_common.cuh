@@ -524,6 +524,9 @@ struct MagnitudeSplit {
 };
 MagnitudeSplit magnitude_split(int64_t m, int64_t n, int64_t k_pad, void* scratch, size_t scratch_bytes,
                                bool only_if_faster);
+MagnitudeSplit magnitude_sums(int64_t m, int64_t n, void* scratch);
+cudaError_t launch_plus_one_rowmax(const float* U, int64_t m, int64_t n, int64_t ldu, float* urow, Oz2Device* dev,
+                                   cudaStream_t st);
 // With `split` the sums are zeroed along the way.
 cudaError_t launch_magnitude_planes(int64_t m, int64_t n, int64_t k, const double* A,
                                     int64_t lda, const double* B, int64_t ldb, const int32_t* ra,
@@ -601,6 +604,11 @@ cudaError_t launch_short_gemm(int64_t m, int64_t n, int64_t k, int64_t c0, int64
 // `scratch` holds the skinny operand's digits and the parts of the sums;
 // `planes` are the digit planes the residue path would store.
 bool skinny_applies(int64_t m, int64_t n, int64_t k, int planes, size_t scratch_bytes);
+// The "+1" pass of a C with few columns, A's magnitude codes formed on chip too.
+bool skinny_plus_one_applies(int64_t m, int64_t n, int64_t k);
+cudaError_t launch_skinny_plus_one(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const int32_t* ra,
+                                   const uint8_t* row_flag, const uint8_t* codes, const MagnitudeSplit& split,
+                                   float* urow, Oz2Device* dev, cudaStream_t st);
 cudaError_t launch_skinny(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B, int64_t ldb,
                           const int32_t* ra, const int32_t* cb, const int32_t* d, const int32_t* e,
                           const uint8_t* row_flag, const uint8_t* col_flag, uint8_t* scratch, double* C, int64_t ldc,

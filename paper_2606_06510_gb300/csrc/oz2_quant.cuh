@@ -70,6 +70,44 @@ __device__ __forceinline__ unsigned long long quantise_tz(double x, int d) {
           (static_cast<uint32_t>(q) ^ sgn)) + (sgn & 1u);
 }
 
+// ⌈log2 |v|⌉ for finite nonzero v.
+__device__ __forceinline__ int ceil_log2_abs(const Split& s) {
+  int bl = 64 - __clzll(static_cast<long long>(s.M));
+  bool pow2 = (s.M & (s.M - 1)) == 0;
+  return s.ex + (pow2 ? bl - 1 : bl);
+}
+
+// E4M3 code of 2^q, q ∈ [-9, 0] (subnormal below 2^-6).
+__device__ __forceinline__ uint32_t e4m3_pow2(int q) {
+  return q >= -6 ? static_cast<uint32_t>((q + 7) << 3) : (1u << (q + 9));
+}
+
+// Magnitude-plane code of x: 0 for x = 0, else the E4M3 code of
+// 2^max(-c, ⌈log2|x|⌉ - ex).  A normal double has ⌈log2|x|⌉ = E - 1023, plus
+// one when its fraction is nonzero, read off the high word; subnormals take
+// the general path.
+__device__ __forceinline__ uint32_t magnitude_code(double x, int ex, int c) {
+  const unsigned long long b = __double_as_longlong(x);
+  const uint32_t hi = static_cast<uint32_t>(b >> 32), lo = static_cast<uint32_t>(b);
+  const int E = static_cast<int>((hi >> 20) & 0x7FFu);
+  const bool frac = ((hi & 0xFFFFFu) | lo) != 0;
+  if (E == 0x7FF) return 0u;  // non-finite entries only occur in rows zeroed by the flags
+  if (E == 0) {
+    if (!frac) return 0u;
+    const Split sp = split_double(x);
+    return e4m3_pow2(max(-c, ceil_log2_abs(sp) - ex));
+  }
+  return e4m3_pow2(max(-c, E - 1023 + (frac ? 1 : 0) - ex));
+}
+
+// The clamp c of the magnitude planes for this k (reading R-scale): the sums of
+// the "+1" GEMM are integers in units of 2^-2c and stay below 2^24.
+inline int magnitude_clamp(int64_t k) {
+  const int lk = k <= 1 ? 0 : 64 - __builtin_clzll(static_cast<unsigned long long>(k - 1));
+  const int c = (24 - lk) / 2;
+  return c < 0 ? 0 : (c > kMagClampMax ? kMagClampMax : c);
+}
+
 // Ã of an entry as a 64-bit two's complement word, any scale and quantiser.
 __device__ __forceinline__ unsigned long long quantise_entry(double x, int d, bool rn) {
   if (!rn && d <= kTzFastMaxD) return quantise_tz(x, d);

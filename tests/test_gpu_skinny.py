@@ -89,6 +89,23 @@ def test_host_column_blocks(oz):
     assert np.array_equal(oz.oz2_dgemm_host(A, B), want.cpu().numpy())
 
 
+@pytest.mark.parametrize("m,n,k", [(4100, 33, 4095), (130, 80, 130000), (16800, 3, 1001)])
+def test_plus_one_pass_on_chip(oz, m, n, k):
+    """A larger than L2 (2^24 entries): its magnitude codes are formed on chip as
+    well.  Rows that are zero, flagged or far down in scale, an odd ld."""
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(97)
+    A = torch.randn((k, m + 1), dtype=torch.float64, device="cuda", generator=g).t()[:m]
+    B = torch.randn((n, k), dtype=torch.float64, device="cuda", generator=g).t()
+    A[5] = 0.0
+    A[7] *= 2.0 ** 300
+    A[9, 3] = float("inf")
+    A[11] *= 2.0 ** -90
+    B[:, 1] = 0.0
+    check(oz, A, B, 12)
+
+
 def test_subnormal_operands(oz):
     A = np.array(wl.random_matrix(150, 400, 1.0, 95)) * 2.0 ** -1060
     B = np.array(wl.random_matrix(400, 20, 1.0, 96)) * 2.0 ** 1000
