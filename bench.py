@@ -459,7 +459,7 @@ def run_oz2(args):
     run_mhz = clk.get("sm_mhz")
     roofline = {"bound": "tensor", "achieved": round(achieved, 1), "peak": round(fp8_peak, 1), "unit": "TFLOP/s",
                 "frac": round(achieved / fp8_peak, 4), "traffic": gemm_traffic(w, r),
-                "kernel": "plane_gemm_kernel<0, 0> (residue GEMM, 3r FP8 plane products)",
+                "kernel": "residue_gemm_kernel (residue GEMM, 3r FP8 plane products)",
                 "peak_source": f"measured fp8 burst: the library's tensor-pipe probe (the GEMM's own MMA, "
                                f"back to back) at SM {probe_mhz} MHz; timed region at SM {run_mhz} MHz",
                 "frac_clock_normalised": (round(achieved / (fp8_peak * run_mhz / probe_mhz), 4)

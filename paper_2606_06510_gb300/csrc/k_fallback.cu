@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(256) fma_gemm_kernel(int64_t m, int64_t n, int
   __shared__ double As[kFK][kFT + 1];
   __shared__ double Bs[kFK][kFT + 1];
   __shared__ int rid[kFT], cid[kFT];
+  pdl_wait();
   if (gridDim.y == 2) {
     if (blockIdx.y == 0) {
       col_list = nullptr;
@@ -134,28 +135,31 @@ static int fb_grid() {
 }
 
 // scratch: (m + n + 2) ints of device memory (counts, then the lists); the
-// two counts must be zero on entry unless `zero_counts` is set.
+// two counts must be zero on entry unless `zero_counts` is set.  With `listed`
+// the flags kernel has filled it (launch_scan_flags).
 cudaError_t launch_fallback_lists(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
                                   int64_t ldb, const uint8_t* row_flag, const uint8_t* col_flag, int* scratch,
-                                  double* C, int64_t ldc, cudaStream_t st, bool zero_counts) {
+                                  double* C, int64_t ldc, cudaStream_t st, bool zero_counts, bool listed) {
   if (m == 0 || n == 0) return cudaSuccess;
   int* counts = scratch;              // [0]: rows, [1]: cols
   int* rlist = scratch + 2;
   int* clist = rlist + m;
-  if (zero_counts) {
-    const cudaError_t err = cudaMemsetAsync(counts, 0, 2 * sizeof(int), st);
+  if (!listed) {
+    if (zero_counts) {
+      const cudaError_t err = cudaMemsetAsync(counts, 0, 2 * sizeof(int), st);
+      if (err != cudaSuccess) return err;
+    }
+    count_launch();
+    const int64_t most = m > n ? m : n;
+    const unsigned cg = static_cast<unsigned>(std::min<int64_t>((most + 255) / 256, 4096));
+    const cudaError_t err = launch_dependent(compact_flags_kernel, dim3(cg, 2), dim3(256), 0, st, m, n, row_flag,
+                                             col_flag, rlist, clist, counts);
     if (err != cudaSuccess) return err;
   }
-  count_launch(2);
-  const int64_t most = m > n ? m : n;
-  const unsigned cg = static_cast<unsigned>(std::min<int64_t>((most + 255) / 256, 4096));
-  const cudaError_t err =
-      launch_dependent(compact_flags_kernel, dim3(cg, 2), dim3(256), 0, st, m, n, row_flag, col_flag, rlist, clist, counts);
-  if (err != cudaSuccess) return err;
   // flagged rows × all columns (blockIdx.y = 0), all rows × flagged columns (1)
-  fma_gemm_kernel<<<dim3(fb_grid(), 2), 256, 0, st>>>(m, n, k, A, lda, B, ldb, rlist, counts, clist, counts + 1, C,
-                                                       ldc);
-  return cudaGetLastError();
+  count_launch();
+  return launch_dependent(fma_gemm_kernel, dim3(fb_grid(), 2), dim3(256), 0, st, m, n, k, A, lda, B, ldb, rlist,
+                          counts, clist, counts + 1, C, ldc);
 }
 
 cudaError_t launch_native(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,

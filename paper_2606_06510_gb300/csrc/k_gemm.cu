@@ -36,7 +36,8 @@
 //
 // Two kernels share this: residue_gemm_kernel (k > 128), which orders a
 // unit's products so that each accumulator is drained while the tensor cores
-// work on the other one, and plane_gemm_kernel, for the one-k-block residue
+// work on the other one (and which has a 64-column form for a C of less than
+// one wave of those tiles), and plane_gemm_kernel, for the one-k-block residue
 // GEMM and the magnitude GEMM, whose units are over before such an overlap
 // could start or use one accumulator only.
 #include <algorithm>
@@ -957,6 +958,10 @@ constexpr int64_t kMinPartSteps = 4;   // k-blocks (512 k-entries) per part at l
 // about 5 TB/s, and a launch).  The pairs' loads are piecewise constant in
 // the pair index, changing only where the heavy units and all units end in
 // their last waves, so those pairs and the two ends cover the maximum.
+// This is the model that oz2_plan reports and that oz2_dgemm_ex's workspace
+// and its callers' saved plans follow; residue_gemm_kernel itself now hides
+// most of a drain and takes the same time for either kind of modulus, which
+// fastest_kparts below goes by.
 static double split_cost(int64_t ntiles, int r, int nsq, int64_t ksteps, int64_t kparts, int64_t pairs, int64_t m,
                          int64_t n) {
   const int64_t s = (ksteps + kparts - 1) / kparts;
@@ -1019,8 +1024,8 @@ int64_t residue_gemm_kparts(int64_t m, int64_t n, int64_t k_pad, int r, int nsq,
 // estimate of this kernel, where a unit's time is its k-blocks (0.96 µs each,
 // every modulus alike) and about three more, and the fold moves the partial
 // residues at 5 TB/s; no split for less than a twentieth.  (1024²×65536, r =
-// 12: 192 units of 512 k-blocks in three waves or 960 of 103
-// in thirteen: 2.79 and 2.72 ms a call; 900×800×40000 r = 10 1.42 and 1.38.)
+// 12: 192 units of 512 k-blocks in three waves or 960 of 103 in thirteen:
+// 2.79 and 2.72 ms a call; 900×800×40000 r = 10 1.42 and 1.38.)
 static int64_t fastest_kparts(int64_t ntiles, int r, int64_t ksteps, int64_t pairs, int64_t m, int64_t n,
                               int64_t max_parts) {
   constexpr double kBlock = 0.96, kUnit = 3.0;  // µs per k-block; a unit's overhead in k-blocks

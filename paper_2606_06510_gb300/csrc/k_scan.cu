@@ -110,7 +110,11 @@ __global__ void __launch_bounds__(256) scan_kernel(int64_t m, int64_t n, int64_t
 // One block per operand (block b takes operand first_op + b; 0: rows of A,
 // 1: columns of B).  Decodes the scan keys, finds the lower median of the exponents of the nonzero finite rows,
 // and writes the flags (bit0: native fallback; bit1: zero in the emulation)
-// and the final exponent (0 for rows that are zero in the emulation).
+// and the final exponent (0 for rows that are zero in the emulation).  With
+// `lists` (two zeroed counts, then room for m rows and n columns) the flagged
+// rows and columns are listed as well, which saves the fallback the launch
+// that lists them (with its own launch as a dependent: 256³ 36.8 → 34.0 µs,
+// 1000×777×1333 115.6 → 111.2, 2048³ at r = 8 255.3 → 251.8).
 constexpr int kExpBins = 2112;   // frexp exponents of finite doubles: [-1073, 1024]
 constexpr int kExpBias = 1080;
 constexpr int kFinalizeThreads = 1024;
@@ -119,7 +123,7 @@ constexpr int kBinsPerThread = (kExpBins + kFinalizeThreads - 1) / kFinalizeThre
 __global__ void __launch_bounds__(kFinalizeThreads) finalize_flags_kernel(int64_t m, int64_t n, int* __restrict__ ra,
                                       int* __restrict__ cb, uint8_t* __restrict__ row_flag,
                                       uint8_t* __restrict__ col_flag, unsigned flags,
-                                      Oz2Device* dev, int first_op) {
+                                      Oz2Device* dev, int first_op, int* __restrict__ lists) {
   __shared__ int hist[kExpBins];
   __shared__ int warp_sum[32];
   __shared__ int med_s;
@@ -210,6 +214,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) finalize_flags_kernel(int64_
       fl[i] = static_cast<uint8_t>((fb ? 1 : 0) | (zero ? 2 : 0));
       key[i] = zero ? 0 : e;
       local += fb ? 1 : 0;
+      if (fb && lists) lists[(is_a ? 2 : 2 + m) + atomicAdd(lists + (is_a ? 0 : 1), 1)] = static_cast<int>(i);
     }
   }
   if (local) atomicAdd(&count_s, local);
@@ -260,25 +265,25 @@ cudaError_t launch_scan_keys(int64_t m, int64_t n, int64_t k, const double* A, i
 }
 
 cudaError_t launch_scan_flags(int64_t m, int64_t n, int ops, unsigned flags, ScanOut out, Oz2Device* dev,
-                              cudaStream_t st) {
+                              cudaStream_t st, int* lists) {
   if ((ops & 3) == 0) return cudaSuccess;
   const int first = (ops & 1) ? 0 : 1;
   const int count = ops == 3 ? 2 : 1;
   count_launch();
   const cudaError_t e = launch_dependent(finalize_flags_kernel, dim3(count), dim3(kFinalizeThreads), 0, st, m, n,
-                                         out.ra, out.cb, out.row_flag, out.col_flag, flags, dev, first);
+                                         out.ra, out.cb, out.row_flag, out.col_flag, flags, dev, first, lists);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_scan(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda,
                         const double* B, int64_t ldb, unsigned flags, ScanOut out,
-                        Oz2Device* dev, cudaStream_t st, bool zero_keys) {
+                        Oz2Device* dev, cudaStream_t st, bool zero_keys, int* lists) {
   cudaError_t err;
   // The scan keys are maxima taken with atomics: zero unless the caller has.
   if (zero_keys && m > 0 && (err = cudaMemsetAsync(out.ra, 0, sizeof(int) * m, st)) != cudaSuccess) return err;
   if (zero_keys && n > 0 && (err = cudaMemsetAsync(out.cb, 0, sizeof(int) * n, st)) != cudaSuccess) return err;
   if ((err = launch_scan_keys(m, n, k, A, lda, B, ldb, out, st, !zero_keys)) != cudaSuccess) return err;
-  return launch_scan_flags(m, n, 3, flags, out, dev, st);
+  return launch_scan_flags(m, n, 3, flags, out, dev, st, lists);
 }
 
 // ---------------------------------------------------------------------------

@@ -20,8 +20,8 @@ cudaError_t launch_scan_keys(int64_t m, int64_t n, int64_t k, const double* A, i
 // Fallback flags and final exponents from complete keys: A's rows when
 // ops & 1, B's columns when ops & 2.  Launched as a programmatic dependent
 // of the kernel before it on the stream (the scan of the operand's last
-// part).
+// part).  With `lists` also the fallback's lists (launch_fallback_lists).
 cudaError_t launch_scan_flags(int64_t m, int64_t n, int ops, unsigned flags, ScanOut out, Oz2Device* dev,
-                              cudaStream_t st);
+                              cudaStream_t st, int* lists = nullptr);
 
 }  // namespace oz2

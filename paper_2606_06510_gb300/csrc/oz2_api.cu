@@ -590,6 +590,10 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
   bool skinny = private_ws && !short_k && skinny_applies(m, n, k, L.num_planes, L.total - L.planes_a);
   for (int b = 0; blocks && b < blocks->count; ++b)
     skinny = skinny && skinny_applies(m, blocks->widths[b], k, L.num_planes, L.total - L.planes_a);
+  // Phase 2 by column blocks (stage timing needs a single block).  In one
+  // block the flags kernel makes the fallback's lists.
+  const bool blocked = blocks && blocks->count > 1 && (flags & OZ2_FLAG_TIMING) == 0;
+  int* lists = private_ws && !blocked ? misc : nullptr;
   int dev = 0;
   cudaGetDevice(&dev);
   HostStats& hs = g_host_stats[dev];
@@ -620,7 +624,7 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
   if (in) {
     if (err == cudaSuccess) err = cudaStreamWaitEvent(s, in->b_ready, 0);
     if (err == cudaSuccess) err = launch_scan_keys(0, n, k, nullptr, lda, B, ldb, so, s);
-    if (err == cudaSuccess) err = launch_scan_flags(m, n, 2, flags, so, ds->status, s);
+    if (err == cudaSuccess) err = launch_scan_flags(m, n, 2, flags, so, ds->status, s, lists);
     if (err == cudaSuccess && scale == OZ2_SCALE_R2)
       err = launch_magnitude_planes(0, n, k, A, lda, B, ldb, ra, cb, rf, cf, mag_a, mag_b, s);
     for (int c = 0; c < in->a_chunks && err == cudaSuccess; ++c) {
@@ -629,9 +633,9 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
       if (err == cudaSuccess)
         err = launch_scan_keys(m, 0, in->a_col0[c + 1] - k0, A + k0 * lda, lda, nullptr, ldb, so, s);
     }
-    if (err == cudaSuccess) err = launch_scan_flags(m, n, 1, flags, so, ds->status, s);
+    if (err == cudaSuccess) err = launch_scan_flags(m, n, 1, flags, so, ds->status, s, lists);
   } else if (err == cudaSuccess) {
-    err = launch_scan(m, n, k, A, lda, B, ldb, flags, so, ds->status, s, false);
+    err = launch_scan(m, n, k, A, lda, B, ldb, flags, so, ds->status, s, false, lists);
   }
   mark(1);
   if (scale == OZ2_SCALE_R2 && skinny && !in && skinny_plus_one_applies(m, n, k)) {
@@ -668,8 +672,6 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
     err = launch_deconstruct(onfly ? 0 : m, n, k, mods, ds->table_a, ds->table_b, A, lda, B, ldb, d, e, rf, cf, quant,
                              pa, pb, s);
   mark(5);
-  // Phase 2 by column blocks (stage timing needs a single block).
-  const bool blocked = blocks && blocks->count > 1 && !ts;
   const int nblk = blocked ? blocks->count : 1;
   int64_t c0 = 0;
   for (int bi = 0; bi < nblk && err == cudaSuccess; ++bi) {
@@ -703,7 +705,7 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
     }
     if (err == cudaSuccess)
       err = launch_fallback_lists(m, cols, k, A, lda, B + c0 * ldb, ldb, rf, cf + c0, misc, C + c0 * ldc, ldc, s,
-                                  c0 > 0);
+                                  c0 > 0, lists != nullptr);
     mark(8);
     if (err == cudaSuccess && on_block) err = (*on_block)(c0, cols);
     c0 += cols;

@@ -514,7 +514,7 @@ struct ScanOut {
 };
 cudaError_t launch_scan(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda,
                         const double* B, int64_t ldb, unsigned flags, ScanOut out,
-                        Oz2Device* dev, cudaStream_t st, bool zero_keys);
+                        Oz2Device* dev, cudaStream_t st, bool zero_keys, int* lists = nullptr);
 // The magnitude GEMM's split along k: its parts (1: none) and the m×n FP32 sums
 // they add into, `count` floats, which must be zero before it runs.
 struct MagnitudeSplit {
@@ -568,7 +568,7 @@ cudaError_t launch_reconstruct(int64_t m, int64_t n, const Oz2Moduli& mods,
 cudaError_t launch_fallback_lists(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda,
                                   const double* B, int64_t ldb, const uint8_t* row_flag,
                                   const uint8_t* col_flag, int* scratch, double* C, int64_t ldc,
-                                  cudaStream_t st, bool zero_counts);
+                                  cudaStream_t st, bool zero_counts, bool listed = false);
 // The tensor-pipe rate probe (k_gemm.cu); reports the CTA pairs it runs on.
 cudaError_t launch_mma_rate(int64_t iters, Oz2Device* dev, int* pairs_out, cudaStream_t st);
 // The fused residue GEMM and reconstruction (k_fused.cu) for r = 11, 12 and
