@@ -34,7 +34,8 @@ __global__ void compact_flags_kernel(int64_t m, int64_t n, const uint8_t* __rest
     if (flag[i] & 1) list[atomicAdd(count + (cols ? 1 : 0), 1)] = static_cast<int>(i);
 }
 
-// rows: row_list ? row_list[0..*row_count) : 0..m-1 ; cols likewise.  With
+// rows: row_list ? row_list[0..*row_count) : 0..m-1 ; cols likewise.  A row list
+// of at most rows_done rows has been dealt with.  With
 // gridDim.y = 2 the blocks with blockIdx.y = 0 take the row list against all
 // columns and those with blockIdx.y = 1 all rows against the column list.
 __global__ void __launch_bounds__(256) fma_gemm_kernel(int64_t m, int64_t n, int64_t k,
@@ -44,7 +45,7 @@ __global__ void __launch_bounds__(256) fma_gemm_kernel(int64_t m, int64_t n, int
                                                        const int* __restrict__ row_count,
                                                        const int* __restrict__ col_list,
                                                        const int* __restrict__ col_count, double* __restrict__ C,
-                                                       int64_t ldc) {
+                                                       int64_t ldc, int rows_done) {
   __shared__ double As[kFK][kFT + 1];
   __shared__ double Bs[kFK][kFT + 1];
   __shared__ int rid[kFT], cid[kFT];
@@ -56,7 +57,7 @@ __global__ void __launch_bounds__(256) fma_gemm_kernel(int64_t m, int64_t n, int
       row_list = nullptr;
     }
   }
-  const int64_t nr = row_list ? *row_count : m;
+  const int64_t nr = !row_list ? m : *row_count <= rows_done ? 0 : *row_count;
   const int64_t nc = col_list ? *col_count : n;
   const int64_t rt = (nr + kFT - 1) / kFT, ct = (nc + kFT - 1) / kFT;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -139,7 +140,8 @@ static int fb_grid() {
 // the flags kernel has filled it (launch_scan_flags).
 cudaError_t launch_fallback_lists(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
                                   int64_t ldb, const uint8_t* row_flag, const uint8_t* col_flag, int* scratch,
-                                  double* C, int64_t ldc, cudaStream_t st, bool zero_counts, bool listed) {
+                                  double* C, int64_t ldc, cudaStream_t st, bool zero_counts, bool listed,
+                                  int rows_done) {
   if (m == 0 || n == 0) return cudaSuccess;
   int* counts = scratch;              // [0]: rows, [1]: cols
   int* rlist = scratch + 2;
@@ -159,14 +161,14 @@ cudaError_t launch_fallback_lists(int64_t m, int64_t n, int64_t k, const double*
   // flagged rows × all columns (blockIdx.y = 0), all rows × flagged columns (1)
   count_launch();
   return launch_dependent(fma_gemm_kernel, dim3(fb_grid(), 2), dim3(256), 0, st, m, n, k, A, lda, B, ldb, rlist,
-                          counts, clist, counts + 1, C, ldc);
+                          counts, clist, counts + 1, C, ldc, rows_done);
 }
 
 cudaError_t launch_native(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
                           int64_t ldb, double* C, int64_t ldc, cudaStream_t st) {
   if (m == 0 || n == 0) return cudaSuccess;
   count_launch();
-  fma_gemm_kernel<<<fb_grid(), 256, 0, st>>>(m, n, k, A, lda, B, ldb, nullptr, nullptr, nullptr, nullptr, C, ldc);
+  fma_gemm_kernel<<<fb_grid(), 256, 0, st>>>(m, n, k, A, lda, B, ldb, nullptr, nullptr, nullptr, nullptr, C, ldc, -1);
   return cudaGetLastError();
 }
 

@@ -24,13 +24,16 @@
 // of 16 KiB at most) stay in shared memory while the CTA walks along its
 // columns; that is what limits k to 64 (the sums stay exact up to 128).
 //
-// Measured on one GB300, 16384²×64, r = 12 (268 M outputs): 2.16 ms for this
+// Flagged rows, when they are few, are recomputed meanwhile by two more warps
+// of every CTA, on the FP64 pipe that nothing else here uses.
+//
+// Measured on one GB300, 16384²×64, r = 12 (268 M outputs): 2.0 ms for this
 // kernel, where the residue GEMM and the reconstruction took 2.47 + 2.02 ms
-// (the call 4.70 → 2.32 ms; k = 32 4.69 → 1.88, k = 16 4.69 → 1.81; r = 6
-// 3.14 → 1.73).  The MMAs alone take 1.45 ms (88 cycles each, the rate of
-// M = 128, N = 176 f16), the epilogue alone 1.6 (some 130 instructions per
-// output); together the tensor pipe is 58% active, its issue slowed by the
-// epilogue warps.
+// (the call 4.70 → 2.15 ms; k = 32 4.69 → 1.75, k = 16 4.69 → 1.66; r = 6
+// 3.14 → 1.54).  The MMAs alone take 1.45 ms (88 cycles each, the rate of
+// M = 128, N = 176 f16), the epilogue alone somewhat more (some 130
+// instructions per output); together the tensor pipe is about 60% active, its
+// issue slowed by the epilogue warps.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -46,13 +49,14 @@ constexpr int kSkDigits = 8;                       // base-256 digits of an inte
 constexpr int kSkK = 64;                           // k-entries of an operand line (128 bytes of f16)
 constexpr int kSkCols = 16;                        // columns of C per tile
 constexpr int kSkClasses = 2 * kSkDigits - 1;      // weights i + j
-constexpr int kSkStages = 4;                       // B tiles in flight
+constexpr int kSkStages = 3;                       // B tiles in flight
 constexpr int kSkGroup = 4;                        // digits of A that share an accumulator window
 constexpr int kSkPad = (kSkGroup - 1) * kSkCols * kPlaneLine;  // zero lines on both sides of a B tile
 constexpr int kSkStageStep = kTileBytes + kSkPad;  // the pad after one tile is the one before the next
 constexpr int kSkBufCols = 256;                    // TMEM columns of an accumulator buffer
 constexpr int kSkEpiWarps = 16;
-constexpr int kSkThreads = 32 * (2 + kSkEpiWarps);  // producer, MMA issuer, epilogue
+constexpr int kSkNativeWarps = 2, kSkNativeRows = 4;
+constexpr int kSkThreads = 32 * (2 + kSkEpiWarps + kSkNativeWarps);  // producer, MMA issuer, epilogue, native FP64
 constexpr int kSkDigitThreads = 1024;              // 128 rows × 8 threads of 8 entries
 static_assert(kSkClasses * kSkCols <= kSkBufCols && 2 * kSkBufCols <= 512, "two buffers in tensor memory");
 static_assert(kSkDigits * kSkCols == kRows, "a B tile is one 128-line block");
@@ -64,6 +68,8 @@ struct ShortArgs {
   const int *d, *e;
   double* C;
   Oz2Device* dev;
+  NativeRows fb;
+  int64_t k;
   int pow256[4];  // 1, 256, 256², 256³: as data, so that the sums stay multiply-adds (as
                   // constants they become shifts and adds, four instructions for one)
 };
@@ -173,6 +179,59 @@ __device__ __forceinline__ DigitCounts digit_counts(int na, int nb) {
   return {a, min(kSkDigits, nb + na + more - a)};
 }
 
+// Flagged rows by FP64 FMA chains in the order of k, as fma_gemm_kernel forms
+// them: a warp takes kSkNativeRows rows × 32 columns, a lane a column, the rows'
+// entries in shared memory.
+__device__ __forceinline__ void native_rows(const ShortArgs& a, int nr, int worker, int workers,
+                                            double (*av)[kSkNativeRows], int lane) {
+  const int64_t chunks = (a.n + 31) / 32, total = (nr + kSkNativeRows - 1) / kSkNativeRows * chunks;
+  const int64_t i1 = total * (worker + 1) / workers;
+  int64_t i = total * worker / workers;
+  int64_t g = i / chunks, c = i - g * chunks, prev = -1;
+  const int k = static_cast<int>(a.k);
+  for (; i < i1; ++i) {
+    if (g != prev) {
+      prev = g;
+      __syncwarp();
+      for (int x = lane; x < k * kSkNativeRows; x += 32) {
+        const int64_t at = g * kSkNativeRows + x % kSkNativeRows;
+        av[x / kSkNativeRows][x % kSkNativeRows] = at < nr ? a.fb.A[a.fb.rows[at] + x / kSkNativeRows * a.fb.lda] : 0.0;
+      }
+      __syncwarp();
+    }
+    const int64_t col = 32 * c + lane;
+    const double* bp = a.fb.B + (col < a.n ? col : a.n - 1) * a.fb.ldb;
+    double acc[kSkNativeRows], b[8];
+#pragma unroll
+    for (int r = 0; r < kSkNativeRows; ++r) acc[r] = 0.0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) b[j] = j < k ? __ldg(bp + j) : 0.0;
+    for (int l0 = 0; l0 < k; l0 += 8) {
+      double next[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) next[j] = l0 + 8 + j < k ? __ldg(bp + l0 + 8 + j) : 0.0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (l0 + j < k) {
+#pragma unroll
+          for (int r = 0; r < kSkNativeRows; ++r) acc[r] = fma(av[l0 + j][r], b[j], acc[r]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) b[j] = next[j];
+    }
+#pragma unroll
+    for (int r = 0; r < kSkNativeRows; ++r) {
+      const int64_t at = g * kSkNativeRows + r;
+      if (at < nr && col < a.n) a.C[a.fb.rows[at] + col * a.ldc] = acc[r];
+    }
+    if (++c == chunks) {
+      c = 0;
+      ++g;
+    }
+  }
+}
+
 // WIDE: |X| may reach 2^127 (r ≥ 14).
 template <bool WIDE>
 __global__ void __launch_bounds__(kSkThreads, 1)
@@ -184,6 +243,7 @@ __global__ void __launch_bounds__(kSkThreads, 1)
   // bars: b_full[4], b_empty[4], acc_full[2], acc_empty[2], a_full, a_empty, drain
   __shared__ uint32_t tmem_base_s;
   __shared__ int na_s, nb_s;
+  __shared__ __align__(16) double native_s[kSkNativeWarps][kSkK][kSkNativeRows];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t bfull = smem_u32(bars), bempty = smem_u32(bars + kSkStages);
   const uint32_t accf = smem_u32(bars + 2 * kSkStages), acce = accf + 16, afull = accf + 32, aempty = accf + 40,
@@ -242,6 +302,8 @@ __global__ void __launch_bounds__(kSkThreads, 1)
   const int nct = static_cast<int>(a.nct);
   const int first_rb = static_cast<int>(t0 / nct), first_ct = static_cast<int>(t0 - static_cast<int64_t>(first_rb) * nct);
   bool ok = true;
+  // Flagged rows that this kernel's FP64 warps take: all of them or none.
+  const int native = a.fb.count && *a.fb.count <= a.fb.most ? *a.fb.count : 0;
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
@@ -353,6 +415,12 @@ __global__ void __launch_bounds__(kSkThreads, 1)
     mma_commit_by(me, drain_bar);  // every MMA retired before the tensor memory goes away
     mbar_wait_bounded(drain_bar, 0, kWaitLimit);
     __syncwarp();
+  } else if (warp >= 2 + kSkEpiWarps) {
+    // ---------------- native FP64 rows ----------------
+    const int w = warp - 2 - kSkEpiWarps;
+    if (native > 0)
+      native_rows(a, native, static_cast<int>(blockIdx.x) * kSkNativeWarps + w, static_cast<int>(gridDim.x) * kSkNativeWarps,
+                  native_s[w], lane);
   } else {
     // ---------------- epilogue ----------------
     // Warps 2..9 take the even tiles (buffer 0), 10..17 the odd ones, so that
@@ -366,12 +434,14 @@ __global__ void __launch_bounds__(kSkThreads, 1)
       int rb = first_rb, ct = first_ct + static_cast<int>(buf), prev = -1;
       uint32_t ph = 0;
       int dr = 0;
+      bool live = false;  // the row exists, and no FP64 warp has it
       for (int64_t t = t0 + buf; t < t1; t += 2, ct += 2, ph ^= 1) {
         for (; ct >= nct; ct -= nct) ++rb;
         const int64_t row = static_cast<int64_t>(rb) * kRows + 32 * q + lane;
         if (rb != prev) {
           prev = rb;
           dr = row < a.m ? __ldg(a.d + row) : 0;
+          live = row < a.m && !(native > 0 && (__ldg(a.fb.flag + row) & 1));
         }
         // The columns' exponents, four ahead of their use (past n: within the
         // array's 256-byte slot).
@@ -382,7 +452,7 @@ __global__ void __launch_bounds__(kSkThreads, 1)
           break;
         }
         tc_fence_after();
-        const bool whole = row < a.m && (ct + 1) * static_cast<int64_t>(kSkCols) <= a.n;
+        const bool whole = live && (ct + 1) * static_cast<int64_t>(kSkCols) <= a.n;
         double* cp = a.C + row + (static_cast<int64_t>(ct) * kSkCols + 8 * h) * a.ldc;
 #pragma unroll 1
         for (int c = 0; c < 8; c += 4) {
@@ -419,7 +489,7 @@ __global__ void __launch_bounds__(kSkThreads, 1)
               val = finish_signed_slow(static_cast<uint32_t>(carry), x[3], x[2], x[1], x[0], E);
             else
               val = finish_signed(x[3], x[2], x[1], x[0], E);
-            if (whole || (row < a.m && col + j < a.n)) *cp = val;
+            if (whole || (live && col + j < a.n)) *cp = val;
             cp += a.ldc;
           }
         }
@@ -479,10 +549,28 @@ cudaError_t launch_short_digits(int64_t m, int64_t n, int64_t k, const double* A
                           xb, mb, k);
 }
 
+static int64_t short_grid(int64_t m, int64_t cols) {
+  return std::min<int64_t>(num_sms(), (m + kRows - 1) / kRows * ((cols + kSkCols - 1) / kSkCols));
+}
+
+// The flagged rows that the FP64 warps take: as many as they finish before the
+// products and the fallback kernel after them would.  Two warps of a CTA run 1 G
+// FMAs a second, the fallback kernel, on all of the FP64 pipe, 0.55 T after 30 µs
+// of its own, and the products 140 G outputs.  16384²×64, a call with 16, 164,
+// 400, 512 flagged rows: 2377, 2707, 3136, 3288 µs with the fallback kernel,
+// 2182, 2198, 2791, 3378 with these warps; 2048²×64 with 64: 140 and 89;
+// 20000×100×64 with 600: 139 and 76; 128²×64 with 1: 69 and 40.
+int short_native_rows(int64_t m, int64_t n, int64_t k) {
+  const double fmas = static_cast<double>((n + 31) / 32 * 32) * static_cast<double>(k);  // a row's, in whole warps
+  const double extra = 1e-9 / static_cast<double>(short_grid(m, n)) - 1 / 0.55e12;
+  const double rows = (static_cast<double>(m) * static_cast<double>(n) / 140e9 + 30e-6) / (fmas * extra);
+  return static_cast<int>(std::min(rows, 1e6));
+}
+
 // Columns [c0, c0 + cols) of C (c0 a multiple of 128; C, e at column c0).
 cudaError_t launch_short_gemm(int64_t m, int64_t n, int64_t k, int64_t c0, int64_t cols, int T, const uint8_t* scratch,
-                              const int32_t* d, const int32_t* e, double* C, int64_t ldc, Oz2Device* dev,
-                              cudaStream_t st) {
+                              const int32_t* d, const int32_t* e, double* C, int64_t ldc, const NativeRows& fb,
+                              Oz2Device* dev, cudaStream_t st) {
   const ShortScratch sc = short_scratch(m, n);
   ShortArgs a{};
   a.m = m;
@@ -498,6 +586,8 @@ cudaError_t launch_short_gemm(int64_t m, int64_t n, int64_t k, int64_t c0, int64
   a.e = e;
   a.C = C;
   a.dev = dev;
+  a.fb = fb;
+  a.k = k;
   for (int i = 0; i < 4; ++i) a.pow256[i] = 1 << (8 * i);
   CUtensorMap ta, tb;
   if (!make_block_map(&ta, scratch, m, kPlaneLine, kSkDigits) ||
@@ -508,7 +598,7 @@ cudaError_t launch_short_gemm(int64_t m, int64_t n, int64_t k, int64_t c0, int64
   const cudaError_t err = allow_smem(reinterpret_cast<const void*>(kern), smem);
   if (err != cudaSuccess) return err;
   count_launch();
-  const int64_t grid = std::min<int64_t>(num_sms(), a.nrb * a.nct);
+  const int64_t grid = short_grid(m, cols);
   return launch_dependent(kern, dim3(static_cast<unsigned>(grid)), dim3(kSkThreads), smem, st, ta, tb, a);
 }
 

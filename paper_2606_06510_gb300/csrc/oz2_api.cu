@@ -594,6 +594,8 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
   // block the flags kernel makes the fallback's lists.
   const bool blocked = blocks && blocks->count > 1 && (flags & OZ2_FLAG_TIMING) == 0;
   int* lists = private_ws && !blocked ? misc : nullptr;
+  // A few flagged rows are recomputed beside the short-k products.
+  const NativeRows native{lists, misc + 2, rf, short_k && lists ? short_native_rows(m, n, k) : -1, A, B, lda, ldb};
   int dev = 0;
   cudaGetDevice(&dev);
   HostStats& hs = g_host_stats[dev];
@@ -679,7 +681,7 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
     const uint8_t* pb0 = pb + static_cast<size_t>(c0 / kPlaneRows) * (L.k_pad / kPlaneLine) * L.num_planes *
                                   static_cast<size_t>(kPlaneBlock);
     if (short_k) {
-      err = launch_short_gemm(m, n, k, c0, cols, mods.T, pa, d, e + c0, C + c0 * ldc, ldc, ds->status, s);
+      err = launch_short_gemm(m, n, k, c0, cols, mods.T, pa, d, e + c0, C + c0 * ldc, ldc, native, ds->status, s);
     } else if (skinny) {
       err = launch_skinny(m, cols, k, A, lda, B + c0 * ldb, ldb, ra, cb + c0, d, e + c0, rf, cf + c0, pa, C + c0 * ldc,
                           ldc, ds->status, s);
@@ -705,7 +707,7 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
     }
     if (err == cudaSuccess)
       err = launch_fallback_lists(m, cols, k, A, lda, B + c0 * ldb, ldb, rf, cf + c0, misc, C + c0 * ldc, ldc, s,
-                                  c0 > 0, lists != nullptr);
+                                  c0 > 0, lists != nullptr, native.most);
     mark(8);
     if (err == cudaSuccess && on_block) err = (*on_block)(c0, cols);
     c0 += cols;

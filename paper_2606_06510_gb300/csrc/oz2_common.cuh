@@ -515,6 +515,15 @@ struct ScanOut {
 cudaError_t launch_scan(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda,
                         const double* B, int64_t ldb, unsigned flags, ScanOut out,
                         Oz2Device* dev, cudaStream_t st, bool zero_keys, int* lists = nullptr);
+// Flagged rows for a kernel that recomputes them itself when there are at most
+// `most` (count null: never): their list, their flags, and the operands.
+struct NativeRows {
+  const int *count, *rows;
+  const uint8_t* flag;
+  int most;
+  const double *A, *B;
+  int64_t lda, ldb;
+};
 // The magnitude GEMM's split along k: its parts (1: none) and the m×n FP32 sums
 // they add into, `count` floats, which must be zero before it runs.
 struct MagnitudeSplit {
@@ -568,7 +577,7 @@ cudaError_t launch_reconstruct(int64_t m, int64_t n, const Oz2Moduli& mods,
 cudaError_t launch_fallback_lists(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda,
                                   const double* B, int64_t ldb, const uint8_t* row_flag,
                                   const uint8_t* col_flag, int* scratch, double* C, int64_t ldc,
-                                  cudaStream_t st, bool zero_counts, bool listed = false);
+                                  cudaStream_t st, bool zero_counts, bool listed = false, int rows_done = -1);
 // The tensor-pipe rate probe (k_gemm.cu); reports the CTA pairs it runs on.
 cudaError_t launch_mma_rate(int64_t iters, Oz2Device* dev, int* pairs_out, cudaStream_t st);
 // The fused residue GEMM and reconstruction (k_fused.cu) for r = 11, 12 and
@@ -597,8 +606,9 @@ bool short_k_applies(int64_t m, int64_t n, int64_t k, size_t scratch_bytes);
 cudaError_t launch_short_digits(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
                                 int64_t ldb, const int32_t* ra, const int32_t* cb, const int32_t* d, const int32_t* e,
                                 const uint8_t* row_flag, const uint8_t* col_flag, uint8_t* scratch, cudaStream_t st);
+int short_native_rows(int64_t m, int64_t n, int64_t k);
 cudaError_t launch_short_gemm(int64_t m, int64_t n, int64_t k, int64_t c0, int64_t cols, int T, const uint8_t* scratch,
-                              const int32_t* d, const int32_t* e, double* C, int64_t ldc, Oz2Device* dev,
+                              const int32_t* d, const int32_t* e, double* C, int64_t ldc, const NativeRows& fb, Oz2Device* dev,
                               cudaStream_t st);
 // C with few rows or columns from base-256 digits formed on chip (k_skinny.cu);
 // `scratch` holds the skinny operand's digits and the parts of the sums;
