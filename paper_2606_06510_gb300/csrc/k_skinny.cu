@@ -25,7 +25,7 @@
 //
 // Measured on one GB300, 16384×16×16384, r = 12: 0.76 ms for this kernel (2.15
 // GB read once, 0.32 ms at the copy rate) against 2.03 + 1.36 for the planes;
-// the call 4.21 → 1.57 ms.  The converting warps' integer pipe bounds it (62
+// the call 4.21 → 1.57 ms (0.71 with seven digits of A instead of eight).  The converting warps' integer pipe bounds it (62
 // instructions per entry, 60% busy, the loads' latency next: a second chunk in
 // flight spills at the 96 registers 18 warps allow and is slower).
 #include <cuda_fp16.h>
@@ -267,13 +267,16 @@ __global__ void __launch_bounds__(kSnThreads, 1) skinny_kernel(const __grid_cons
     atomicMax(&nb_s, need);
   }
   __syncthreads();
-  // Twelve weights or all fifteen (the digits added are zero).
+  // Thirteen weights, which r = 12 needs, or all fifteen.  The digits added are
+  // zero: the skinny operand's first, since the tall one's are formed here.
+  // (With twelve or fifteen, the tall operand's first, 16384×16×16384 r = 12
+  // 1.433 ms a call against 1.387, 9000×16×9000 r = 6 0.485 against 0.463.)
   int na = na_s, nb = nb_s;
-  if (na + nb - 1 <= 12) {
-    const int more = 13 - na - nb;
-    const int x = min(kSnDigits, na + more);
-    nb += na + more - x;
-    na = x;
+  if (na + nb - 1 <= 13) {
+    const int more = 14 - na - nb;
+    const int x = min(kSnDigits, nb + more);  // the skinny operand's: its tiles hold all eight
+    na += nb + more - x;
+    nb = x;
   } else {
     na = nb = kSnDigits;
   }
@@ -519,7 +522,7 @@ __global__ void __launch_bounds__(kSnThreads, 1) skinny_kernel(const __grid_cons
       }
       if (ok && units > 0) drain(units - 1, out, out_q);
     };
-    if (na + nb - 1 <= 12) run(std::integral_constant<int, 12>());
+    if (na + nb - 1 <= 13) run(std::integral_constant<int, 13>());
     else run(std::integral_constant<int, kSnClasses>());
     if (!ok && lane == 0) {
       a.dev->status = kStatusTimeout;
