@@ -330,7 +330,9 @@ int oz2_scan(int64_t m, int64_t n, int64_t k,
 /* Stage 1b+2' (§2.4, "+1" pass): magnitude planes Â_il = 2^max(-c, ⌈log2
  * |A_il|2^-ra_i⌉) (E4M3, m×k_pad and n×k_pad as the digit planes), the
  * FP8 GEMM U = ÂB̂ (exact in FP32), and the exponents d[m], e[n]
- * (oz2_scale_mode).  d_urow receives max_j U_ij.  d_mag_a/d_mag_b are outputs. */
+ * (oz2_scale_mode).  d_urow receives max_j U_ij.  d_mag_a/d_mag_b are outputs.
+ * With R2 it allocates and frees one word stream-ordered (max_ij U_ij, which
+ * every call keeps for itself: calls on several streams may overlap). */
 int oz2_scale(int64_t m, int64_t n, int64_t k, int num_moduli,
               const double* d_A, int64_t lda, const double* d_B, int64_t ldb,
               const int32_t* d_ra, const int32_t* d_cb,

@@ -60,6 +60,7 @@ constexpr int kGroupM = 8;                       // tile rasterisation group
 struct EpiCtx {
   int16_t* res;   // r × (m×n column-major, ld = ldr ≥ m; matrix i at i·n·ldr)
   float* urow;
+  int* u_max;     // float bits of max_ij U_ij
   Oz2Device* dev;
   int64_t m, n, ldr;
   float* upart;   // magnitude GEMM split along k: U (m×n row-major, ld = ldu) summed over the parts
@@ -392,7 +393,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         // rows past m hold zeros (TMA fills out-of-range rows with 0)
         if (row < ctx.m) atomicMax(reinterpret_cast<int*>(ctx.urow) + row, __float_as_int(rowmax));
         const int wm = __reduce_max_sync(0xffffffffu, __float_as_int(rowmax));
-        if (lane == 0) atomicMax(&ctx.dev->u_max_bits, wm);
+        if (lane == 0) atomicMax(ctx.u_max, wm);
       }
     }
     if (!ok) {
@@ -832,7 +833,7 @@ __global__ void plane_gemm_simt_kernel(const uint8_t* __restrict__ pa, const uin
     float acc = 0.f;
     for (int64_t l = 0; l < k_pad; ++l) acc += e4m3_to_float(ar[l]) * e4m3_to_float(bc[l]);
     atomicMax(reinterpret_cast<int*>(ctx.urow) + row, __float_as_int(acc));
-    atomicMax(&ctx.dev->u_max_bits, __float_as_int(acc));
+    atomicMax(ctx.u_max, __float_as_int(acc));
     return;
   }
   for (int i = 0; i < mods.r; ++i) {
@@ -1055,7 +1056,7 @@ static size_t gemm_smem_bytes() { return 1024 + static_cast<size_t>(kStages) * k
 constexpr int kRowMaxThreads = 256;
 __global__ void __launch_bounds__(kRowMaxThreads) plus_one_rowmax_kernel(const float* __restrict__ U, int64_t m,
                                                                          int64_t n, int64_t ldu,
-                                                                         float* __restrict__ urow, Oz2Device* dev) {
+                                                                         float* __restrict__ urow, int* u_max) {
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int64_t row = static_cast<int64_t>(blockIdx.x) * (kRowMaxThreads / 32) + (threadIdx.x >> 5);
@@ -1066,16 +1067,16 @@ __global__ void __launch_bounds__(kRowMaxThreads) plus_one_rowmax_kernel(const f
   const int wm = __reduce_max_sync(0xffffffffu, __float_as_int(mx));  // nonnegative floats order as their bits
   if (lane == 0) {
     atomicMax(reinterpret_cast<int*>(urow) + row, wm);
-    atomicMax(&dev->u_max_bits, wm);
+    atomicMax(u_max, wm);
   }
 }
 
-cudaError_t launch_plus_one_rowmax(const float* U, int64_t m, int64_t n, int64_t ldu, float* urow, Oz2Device* dev,
+cudaError_t launch_plus_one_rowmax(const float* U, int64_t m, int64_t n, int64_t ldu, float* urow, int* u_max,
                                    cudaStream_t st) {
   constexpr int64_t rows_per_block = kRowMaxThreads / 32;
   count_launch();
   return launch_dependent(plus_one_rowmax_kernel, dim3(static_cast<unsigned>((m + rows_per_block - 1) / rows_per_block)),
-                          dim3(kRowMaxThreads), 0, st, U, m, n, ldu, urow, dev);
+                          dim3(kRowMaxThreads), 0, st, U, m, n, ldu, urow, u_max);
 }
 
 // The sums of a magnitude GEMM that adds into U anyway (k_skinny.cu).
@@ -1207,10 +1208,10 @@ int64_t resident_pairs(const void* kernel, int threads, size_t smem) {
 //       2 residues (SIMT reference), 3 magnitude (SIMT reference).
 cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Moduli& mods,
                               const uint8_t* planes_a, const uint8_t* planes_b, int mode,
-                              int16_t* residues, int64_t ldr, float* urow, Oz2Device* dev, cudaStream_t st,
-                              int16_t* partials, size_t partial_bytes, const MagnitudeSplit* split, bool fastest) {
+                              int16_t* residues, int64_t ldr, float* urow, int* u_max, Oz2Device* dev,
+                              cudaStream_t st, int16_t* partials, size_t partial_bytes, const MagnitudeSplit* split, bool fastest) {
   if (m == 0 || n == 0) return cudaSuccess;
-  EpiCtx ctx{residues, urow, dev, m, n, ldr, nullptr, 0};
+  EpiCtx ctx{residues, urow, u_max, dev, m, n, ldr, nullptr, 0};
   if (mode >= 2) {
     dim3 g(static_cast<unsigned>((m + 127) / 128), static_cast<unsigned>(n));
     count_launch();
@@ -1290,7 +1291,7 @@ cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Modu
   // 1024²×65536 2795 and 2873).
   err = launch_dependent(kern, dim3(static_cast<unsigned>(2 * pairs)), dim3(kGemmThreads), smem, st, ta, tb, mods, k_pad,
                          um, ctx);
-  if (err == cudaSuccess && ctx.upart) err = launch_plus_one_rowmax(ctx.upart, m, n, ctx.ldu, urow, dev, st);
+  if (err == cudaSuccess && ctx.upart) err = launch_plus_one_rowmax(ctx.upart, m, n, ctx.ldu, urow, u_max, st);
   if (err == cudaSuccess && mode == 0 && um.kparts > 1) {  // the residue GEMM's parts, folded into C^(i)
     const int64_t row_threads = (m + 7) / 8;
     dim3 g(static_cast<unsigned>((row_threads + kFoldThreads - 1) / kFoldThreads),

@@ -297,8 +297,8 @@ __device__ __forceinline__ int ceil_log2_f32(float u) {
 }
 
 __global__ void choose_scales_kernel(int64_t m, int64_t n, int64_t k, int T, int scale_mode,
-                                     const float* __restrict__ urow, const int* __restrict__ ra,
-                                     const int* __restrict__ cb,
+                                     const float* __restrict__ urow, const int* u_max,
+                                     const int* __restrict__ ra, const int* __restrict__ cb,
                                      const uint8_t* __restrict__ row_flag,
                                      const uint8_t* __restrict__ col_flag, int* __restrict__ d,
                                      int* __restrict__ e, Oz2Device* dev) {
@@ -307,7 +307,9 @@ __global__ void choose_scales_kernel(int64_t m, int64_t n, int64_t k, int T, int
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   int s, umax = 0;
   if (scale_mode == OZ2_SCALE_R2) {
-    float ug = __int_as_float(dev->u_max_bits);
+    const int bits = *u_max;
+    const float ug = __int_as_float(bits);
+    if (idx == 0) dev->u_max_bits = bits;
     umax = ug > 0.f ? ceil_log2_f32(ug) : 0;
     s = min(62, (T - umax) >> 1);
   } else {
@@ -336,7 +338,7 @@ __global__ void choose_scales_kernel(int64_t m, int64_t n, int64_t k, int T, int
 }
 
 cudaError_t launch_choose_scales(int64_t m, int64_t n, int64_t k, const Oz2Moduli& mods,
-                                 int scale_mode, const float* urow, const int32_t* ra,
+                                 int scale_mode, const float* urow, const int* u_max, const int32_t* ra,
                                  const int32_t* cb, const uint8_t* row_flag,
                                  const uint8_t* col_flag, int32_t* d, int32_t* e,
                                  Oz2Device* dev, cudaStream_t st) {
@@ -344,7 +346,7 @@ cudaError_t launch_choose_scales(int64_t m, int64_t n, int64_t k, const Oz2Modul
   if (tot == 0) return cudaSuccess;
   count_launch();
   return launch_dependent(choose_scales_kernel, dim3(static_cast<unsigned>((tot + 255) / 256)), dim3(256), 0, st, m, n,
-                          k, mods.T, scale_mode, urow, ra, cb, row_flag, col_flag, d, e, dev);
+                          k, mods.T, scale_mode, urow, u_max, ra, cb, row_flag, col_flag, d, e, dev);
 }
 
 }  // namespace oz2

@@ -828,7 +828,7 @@ bool skinny_plus_one_applies(int64_t m, int64_t n, int64_t k) { return n <= m &&
 // 4) and its row maxima.  `codes` are B's magnitude codes.
 cudaError_t launch_skinny_plus_one(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const int32_t* ra,
                                    const uint8_t* row_flag, const uint8_t* codes, const MagnitudeSplit& split,
-                                   float* urow, Oz2Device* dev, cudaStream_t st) {
+                                   float* urow, int* u_max, Oz2Device* dev, cudaStream_t st) {
   SkinnyPlusArgs a{};
   a.A = A;
   a.lda = lda;
@@ -854,7 +854,7 @@ cudaError_t launch_skinny_plus_one(int64_t m, int64_t n, int64_t k, const double
   count_launch();
   const int64_t grid = std::min<int64_t>(2 * num_sms(), a.total);
   err = launch_dependent(skinny_plus_one_kernel, dim3(static_cast<unsigned>(grid)), dim3(kSpThreads), smem, st, a);
-  return err != cudaSuccess ? err : launch_plus_one_rowmax(split.sums, m, n, a.ldu, urow, dev, st);
+  return err != cudaSuccess ? err : launch_plus_one_rowmax(split.sums, m, n, a.ldu, urow, u_max, st);
 }
 
 cudaError_t launch_skinny(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B, int64_t ldb,

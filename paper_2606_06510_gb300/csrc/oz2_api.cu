@@ -22,6 +22,7 @@ static const int kModuliAll[kMaxModuli] = {1089, 1024, 961, 841, 625, 529, 511, 
 constexpr int kTableMax = 20480;  // 2·Σ of the ten nonsquare moduli = 9740 entries
 constexpr int kHostBlocksMax = 8;   // column blocks of one oz2_dgemm_host call
 constexpr int kHostAChunksMax = 4;  // column chunks A is copied in by oz2_dgemm_host
+constexpr size_t kPrivateBytes = 256;  // past the layout, in a workspace the library allocates itself
 
 // Packed E4M3 digit planes of every residue (byte p = plane p) of the
 // nonsquare moduli, 2m entries per modulus, entry i for the residue
@@ -388,15 +389,17 @@ __global__ void reset_status_kernel(Oz2Device* dev) {
 
 // The start of a call: the status summary, and the workspace words that
 // later stages accumulate with atomics (scan keys ra, cb; the "+1" row
-// maxima; the two fallback counts) set to zero, in one launch.
+// maxima and their maximum; the two fallback counts) set to zero, in one
+// launch.
 __global__ void prepare_call_kernel(Oz2Device* dev, int* ra, int64_t m, int* cb, int64_t n, float* urow,
-                                    int* counts) {
+                                    int* u_max, int* counts) {
   pdl_trigger();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     dev->fallback_rows = 0;
     dev->fallback_cols = 0;
     dev->u_max_bits = 0;
     dev->s = 0;
+    *u_max = 0;
     counts[0] = 0;
     counts[1] = 0;
   }
@@ -553,7 +556,7 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
 
   oz2_ws_layout L;
   compute_layout(m, n, k, num_moduli, &L);
-  if (!workspace || ws_bytes < L.total || (reinterpret_cast<uintptr_t>(workspace) & 255)) return OZ2_ERR_ALLOC;
+  if (!workspace || ws_bytes < L.total + (private_ws ? kPrivateBytes : 0) || (reinterpret_cast<uintptr_t>(workspace) & 255)) return OZ2_ERR_ALLOC;
   DeviceState* ds = nullptr;
   if ((st = device_state(&ds)) != OZ2_OK) return st;
   const Oz2Moduli& mods = moduli_for(num_moduli, quant);
@@ -567,6 +570,11 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
   int32_t* e = reinterpret_cast<int32_t*>(ws + L.e);
   float* urow = reinterpret_cast<float*>(ws + L.urow);
   int* misc = reinterpret_cast<int*>(ws + L.misc);
+  // max_ij U_ij of the "+1" pass, which the scales depend on: a word of this
+  // call's own, since calls on several streams overlap.  It is the first entry
+  // of the fallback's lists, which are made when the scales are long chosen,
+  // or, where the flags kernel may make them before, past the layout.
+  int* u_max = private_ws ? reinterpret_cast<int*>(ws + L.total) : misc + 2;
   uint8_t* mag_a = ws + L.mag_a;
   uint8_t* mag_b = ws + L.mag_b;
   uint8_t* pa = ws + L.planes_a;
@@ -619,7 +627,7 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
   {
     const int64_t blocks = std::min<int64_t>((m + n + 255) / 256, 1024);
     prepare_call_kernel<<<static_cast<unsigned>(std::max<int64_t>(blocks, 1)), 256, 0, s>>>(ds->status, ra, m, cb,
-                                                                                              n, urow, misc);
+                                                                                              n, urow, u_max, misc);
   }
   mark(0);
   const ScanOut so{ra, cb, rf, cf};
@@ -646,7 +654,7 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
     if (err == cudaSuccess) err = launch_magnitude_planes(0, n, k, A, lda, B, ldb, ra, cb, rf, cf, mag_a, mag_b, s, &sums);
     mark(2);
     if (err == cudaSuccess)
-      err = launch_skinny_plus_one(m, n, k, A, lda, ra, rf, mag_b, sums, urow, ds->status, s);
+      err = launch_skinny_plus_one(m, n, k, A, lda, ra, rf, mag_b, sums, urow, u_max, ds->status, s);
     mark(3);
   } else if (scale == OZ2_SCALE_R2) {
     // The digit-plane and residue regions are not yet in use: the scratch for
@@ -658,14 +666,14 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
       err = launch_magnitude_planes(m, in ? 0 : n, k, A, lda, B, ldb, ra, cb, rf, cf, mag_a, mag_b, s, &split);
     mark(2);
     if (err == cudaSuccess)
-      err = launch_plane_gemm(m, n, L.k_pad, mods, mag_a, mag_b, simt ? 3 : 1, nullptr, 0, urow, ds->status, s, nullptr, 0,
-                              &split);
+      err = launch_plane_gemm(m, n, L.k_pad, mods, mag_a, mag_b, simt ? 3 : 1, nullptr, 0, urow, u_max, ds->status, s,
+                              nullptr, 0, &split);
     mark(3);
   } else {
     mark(2);
     mark(3);
   }
-  if (err == cudaSuccess) err = launch_choose_scales(m, n, k, mods, scale, urow, ra, cb, rf, cf, d, e, ds->status, s);
+  if (err == cudaSuccess) err = launch_choose_scales(m, n, k, mods, scale, urow, u_max, ra, cb, rf, cf, d, e, ds->status, s);
   mark(4);
   if (short_k) {
     if (err == cudaSuccess)
@@ -696,7 +704,7 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
       } else {
         // The magnitude planes are dead once the scales are chosen: their
         // region is the scratch for the partial residues of a split-K GEMM.
-        err = launch_plane_gemm(m, cols, L.k_pad, mods, pa, pb0, simt ? 2 : 0, res, L.res_ld, nullptr, ds->status, s,
+        err = launch_plane_gemm(m, cols, L.k_pad, mods, pa, pb0, simt ? 2 : 0, res, L.res_ld, nullptr, nullptr, ds->status, s,
                                 reinterpret_cast<int16_t*>(mag_a), L.planes_a - L.mag_a, nullptr,
                                 private_ws && !blocked);
       }
@@ -889,7 +897,7 @@ int oz2_dgemm(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, con
     return oz2_dgemm_ex(m, n, k, A, lda, B, ldb, C, ldc, num_moduli, OZ2_QUANT_TZ, OZ2_SCALE_R2, 0, nullptr, 0,
                         stream);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  size_t bytes = oz2_workspace_size(m, n, k, num_moduli);
+  size_t bytes = oz2_workspace_size(m, n, k, num_moduli) + kPrivateBytes;
   void* ws = nullptr;
   if (pool_alloc(&ws, bytes, s) != cudaSuccess) {
     cudaGetLastError();
@@ -926,7 +934,7 @@ int oz2_dgemm_host(int64_t m, int64_t n, int64_t k, const double* hA, int64_t ld
   cudaStream_t cs = ds->copy_stream;
   const size_t bA = align256(sizeof(double) * m * k), bB = align256(sizeof(double) * k * n),
                bC = align256(sizeof(double) * m * n);
-  const size_t ws = k > 0 ? oz2_workspace_size(m, n, k, num_moduli) : 0;
+  const size_t ws = k > 0 ? oz2_workspace_size(m, n, k, num_moduli) + kPrivateBytes : 0;
   uint8_t* buf = nullptr;
   if (pool_alloc(reinterpret_cast<void**>(&buf), bA + bB + bC + ws, s) != cudaSuccess) {
     cudaGetLastError();
@@ -1117,17 +1125,24 @@ int oz2_scale(int64_t m, int64_t n, int64_t k, int num_moduli, const double* A, 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const Oz2Moduli& mods = moduli_for(num_moduli, quant);
   const int64_t k_pad = (k + kKPad - 1) / kKPad * kKPad;
+  int* u_max = nullptr;  // the call's own word (run_stages)
+  if (scale == OZ2_SCALE_R2 && pool_alloc(reinterpret_cast<void**>(&u_max), sizeof(int), s) != cudaSuccess) {
+    cudaGetLastError();
+    return OZ2_ERR_ALLOC;
+  }
   count_launch();
   reset_status_kernel<<<1, 1, 0, s>>>(ds->status);
   cudaError_t err = cudaMemsetAsync(urow, 0, sizeof(float) * m, s);
   if (scale == OZ2_SCALE_R2) {
+    if (err == cudaSuccess) err = cudaMemsetAsync(u_max, 0, sizeof(int), s);
     if (err == cudaSuccess)
       err = launch_magnitude_planes(m, n, k, A, lda, B, ldb, ra, cb, row_flag, col_flag, mag_a, mag_b, s);
     if (err == cudaSuccess)
-      err = launch_plane_gemm(m, n, k_pad, mods, mag_a, mag_b, 1, nullptr, 0, urow, ds->status, s);
+      err = launch_plane_gemm(m, n, k_pad, mods, mag_a, mag_b, 1, nullptr, 0, urow, u_max, ds->status, s);
   }
   if (err == cudaSuccess)
-    err = launch_choose_scales(m, n, k, mods, scale, urow, ra, cb, row_flag, col_flag, d, e, ds->status, s);
+    err = launch_choose_scales(m, n, k, mods, scale, urow, u_max, ra, cb, row_flag, col_flag, d, e, ds->status, s);
+  if (u_max) cudaFreeAsync(u_max, s);
   return to_status(err);
 }
 
@@ -1155,7 +1170,7 @@ int oz2_residue_gemm(int64_t m, int64_t n, int64_t k, int num_moduli, const uint
   if (st) return st;
   const Oz2Moduli& mods = moduli_for(num_moduli, OZ2_QUANT_TZ);
   const int64_t k_pad = (k + kKPad - 1) / kKPad * kKPad;
-  return to_status(launch_plane_gemm(m, n, k_pad, mods, planes_a, planes_b, 0, residues, ldr, nullptr, ds->status,
+  return to_status(launch_plane_gemm(m, n, k_pad, mods, planes_a, planes_b, 0, residues, ldr, nullptr, nullptr, ds->status,
                                      static_cast<cudaStream_t>(stream)));
 }
 
@@ -1168,7 +1183,7 @@ int oz2_residue_gemm_simt(int64_t m, int64_t n, int64_t k, int num_moduli, const
   if (st) return st;
   const Oz2Moduli& mods = moduli_for(num_moduli, OZ2_QUANT_TZ);
   const int64_t k_pad = (k + kKPad - 1) / kKPad * kKPad;
-  return to_status(launch_plane_gemm(m, n, k_pad, mods, planes_a, planes_b, 2, residues, ldr, nullptr, ds->status,
+  return to_status(launch_plane_gemm(m, n, k_pad, mods, planes_a, planes_b, 2, residues, ldr, nullptr, nullptr, ds->status,
                                      static_cast<cudaStream_t>(stream)));
 }
 

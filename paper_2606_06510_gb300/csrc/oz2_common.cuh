@@ -167,7 +167,7 @@ struct Oz2Device {
   int timeout_site;
   int fallback_rows;
   int fallback_cols;
-  int u_max_bits;               // float bits of max_ij U_ij ("+1" pass)
+  int u_max_bits;               // float bits of max_ij U_ij ("+1" pass), for the statistics
   int s;                        // column budget (R2) or pB (R1)
   int pad[10];
 };
@@ -534,7 +534,7 @@ struct MagnitudeSplit {
 MagnitudeSplit magnitude_split(int64_t m, int64_t n, int64_t k_pad, void* scratch, size_t scratch_bytes,
                                bool only_if_faster);
 MagnitudeSplit magnitude_sums(int64_t m, int64_t n, void* scratch);
-cudaError_t launch_plus_one_rowmax(const float* U, int64_t m, int64_t n, int64_t ldu, float* urow, Oz2Device* dev,
+cudaError_t launch_plus_one_rowmax(const float* U, int64_t m, int64_t n, int64_t ldu, float* urow, int* u_max,
                                    cudaStream_t st);
 // With `split` the sums are zeroed along the way.
 cudaError_t launch_magnitude_planes(int64_t m, int64_t n, int64_t k, const double* A,
@@ -543,7 +543,7 @@ cudaError_t launch_magnitude_planes(int64_t m, int64_t n, int64_t k, const doubl
                                     const uint8_t* col_flag, uint8_t* mag_a, uint8_t* mag_b,
                                     cudaStream_t st, const MagnitudeSplit* split = nullptr);
 cudaError_t launch_choose_scales(int64_t m, int64_t n, int64_t k, const Oz2Moduli& mods,
-                                 int scale_mode, const float* urow, const int32_t* ra,
+                                 int scale_mode, const float* urow, const int* u_max, const int32_t* ra,
                                  const int32_t* cb, const uint8_t* row_flag,
                                  const uint8_t* col_flag, int32_t* d, int32_t* e,
                                  Oz2Device* dev, cudaStream_t st);
@@ -564,9 +564,12 @@ int64_t magnitude_gemm_kparts(int64_t m, int64_t n, int64_t k_pad, size_t scratc
 // residue GEMM may split K into (the parts' residues); `split` is the magnitude
 // GEMM's.  Neither may overlap the operands, C^(i) or urow.  With `fastest` the
 // parts are not residue_gemm_kparts' but this library's own best estimate.
+// The magnitude GEMM (modes 1, 3) takes maxima into `urow` and, over all rows,
+// into `u_max` (both zero before it runs, both the call's own).
 cudaError_t launch_plane_gemm(int64_t m, int64_t n, int64_t k_pad, const Oz2Moduli& mods,
                               const uint8_t* planes_a, const uint8_t* planes_b, int mode,
-                              int16_t* residues, int64_t ldr, float* urow, Oz2Device* dev, cudaStream_t st,
+                              int16_t* residues, int64_t ldr, float* urow, int* u_max, Oz2Device* dev,
+                              cudaStream_t st,
                               int16_t* partials = nullptr, size_t partial_bytes = 0,
                               const MagnitudeSplit* split = nullptr, bool fastest = false);
 // `centred`: every residue lies in [-⌊m_k/2⌋, m_k-1-⌊m_k/2⌋] (as the residue
@@ -618,7 +621,7 @@ bool skinny_applies(int64_t m, int64_t n, int64_t k, int planes, size_t scratch_
 bool skinny_plus_one_applies(int64_t m, int64_t n, int64_t k);
 cudaError_t launch_skinny_plus_one(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const int32_t* ra,
                                    const uint8_t* row_flag, const uint8_t* codes, const MagnitudeSplit& split,
-                                   float* urow, Oz2Device* dev, cudaStream_t st);
+                                   float* urow, int* u_max, Oz2Device* dev, cudaStream_t st);
 cudaError_t launch_skinny(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B, int64_t ldb,
                           const int32_t* ra, const int32_t* cb, const int32_t* d, const int32_t* e,
                           const uint8_t* row_flag, const uint8_t* col_flag, uint8_t* scratch, double* C, int64_t ldc,
