@@ -233,7 +233,10 @@ int oz2_workspace_layout(int64_t m, int64_t n, int64_t k, int num_moduli,
  *                 block (its copy is the one left exposed); short k, where
  *                 the copies dominate, a narrow first one (the copies start
  *                 early).  Identical shapes reuse the last plan.
- *   host_kparts   the residue GEMM's kparts for each block.
+ *   host_kparts   the residue GEMM's kparts for each block.  (With k ≤ 64, or
+ *                 few rows or columns of C, oz2_dgemm_host and oz2_dgemm
+ *                 run kernels that form no residues: kparts then holds for
+ *                 oz2_dgemm_ex alone, and host_kparts for no call.)
  *   mag_kparts    parts of k of the "+1" magnitude GEMM (1: no split).
  *                 When its 256×256 tiles fill less than half a wave (a
  *                 small C with a long k), each tile runs in up to 64 parts
@@ -241,8 +244,8 @@ int oz2_workspace_layout(int64_t m, int64_t n, int64_t k, int num_moduli,
  *                 (exact: integers in units of 2^-2c below 2^24) into an
  *                 m×n buffer in the then unused digit-plane region, and a
  *                 row-maximum kernel follows (one launch more).
- *                 oz2_dgemm and oz2_dgemm_host, whose launches nobody
- *                 plans by, make the split only where it is faster.
+ *                 oz2_dgemm and oz2_dgemm_host make the split only where
+ *                 it is faster.
  * Returns OZ2_OK, OZ2_ERR_INVALID_ARG (null out, negative sizes,
  * cta_pairs < 1) or OZ2_ERR_UNSUPPORTED_R. */
 typedef struct {

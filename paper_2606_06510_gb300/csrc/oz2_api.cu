@@ -706,7 +706,7 @@ static int run_stages(int64_t m, int64_t n, int64_t k, const double* A, int64_t 
         // region is the scratch for the partial residues of a split-K GEMM.
         err = launch_plane_gemm(m, cols, L.k_pad, mods, pa, pb0, simt ? 2 : 0, res, L.res_ld, nullptr, nullptr, ds->status, s,
                                 reinterpret_cast<int16_t*>(mag_a), L.planes_a - L.mag_a, nullptr,
-                                private_ws && !blocked);
+                                private_ws && !blocks);  // a host call keeps to oz2_plan's parts
       }
       mark(6);
       if (err == cudaSuccess)
