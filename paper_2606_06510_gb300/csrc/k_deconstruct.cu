@@ -11,7 +11,7 @@
 // rows in flight per block).  A is column-major: the threads of a warp that
 // load the same k-entries read consecutive rows.  B's rows are contiguous in
 // k and are read with 16-byte vector loads.  One launch covers both
-// operands: the first blocks work on A, the rest on B.
+// operands: every block walks A's tiles and then B's.
 #include <algorithm>
 #include <utility>
 

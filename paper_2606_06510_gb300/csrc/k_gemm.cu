@@ -1026,7 +1026,8 @@ int64_t residue_gemm_kparts(int64_t m, int64_t n, int64_t k_pad, int r, int nsq,
 // every modulus alike) and about three more, and the fold moves the partial
 // residues at 5 TB/s; no split for less than a twentieth.  (1024²×65536, r =
 // 12: 192 units of 512 k-blocks in three waves or 960 of 103 in thirteen:
-// 2.79 and 2.72 ms a call; 900×800×40000 r = 10 1.42 and 1.38.)
+// 2.77 and 2.70 ms a call, both in turn; 900×800×40000 r = 10 1.41 and 1.36,
+// 1040×651×47202 r = 8 1.38 and 1.31.)
 static int64_t fastest_kparts(int64_t ntiles, int r, int64_t ksteps, int64_t pairs, int64_t m, int64_t n,
                               int64_t max_parts) {
   constexpr double kBlock = 0.96, kUnit = 3.0;  // µs per k-block; a unit's overhead in k-blocks

@@ -141,32 +141,6 @@ __global__ void __launch_bounds__(kSkDigitThreads) short_digits_kernel(DigitOper
 // ---------------------------------------------------------------------------
 // Digit products and C.
 // ---------------------------------------------------------------------------
-// D[tmem] (+)= A[smem]·B[smem]^T, f16 operands.  The whole warp runs the
-// issuing code and the lane with `me` set issues: descriptors then stay in
-// uniform registers (in one lane's code each had to be moved there, some 130
-// cycles an instruction, which was what a tile took).
-__device__ __forceinline__ void mma_f16(uint32_t me, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                        uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
-      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(me)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit_by(uint32_t me, uint32_t bar) {
-  asm volatile(
-      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
-      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
-      "r"(me)
-      : "memory");
-}
-
-__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
-  long long r;
-  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
-  return r;
-}
-
 // The digit counts a launch runs with, for operands that need na and nb:
 // digits that are all zero make the weights, na + nb - 1, a multiple of four
 // (or all 15), since the epilogue takes them in fours.  They go to B first: a
@@ -243,7 +217,7 @@ __global__ void __launch_bounds__(kSkThreads, 1)
   uint8_t* sm_a = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sm_b = sm_a + kSkDigits * kTileBytes + kSkPad;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm_b + kSkStages * kSkStageStep);
-  // bars: b_full[4], b_empty[4], acc_full[2], acc_empty[2], a_full, a_empty, drain
+  // bars: b_full[kSkStages], b_empty[kSkStages], acc_full[2], acc_empty[2], a_full, a_empty, drain
   __shared__ uint32_t tmem_base_s;
   __shared__ int na_s, nb_s;
   __shared__ __align__(16) double native_s[kSkNativeWarps][kSkK][kSkNativeRows];
@@ -384,17 +358,17 @@ __global__ void __launch_bounds__(kSkThreads, 1)
           const uint32_t acc = acc0 + i0 * kSkCols, all = idesc(nb + gd - 1);
           const uint64_t ag = da + i0 * (kTileBytes >> 4);
           if (i0 == 0) {
-            mma_f16(me, acc, ag, b, all, 0u);
+            mma_f16_by(me, acc, ag, b, all, 0u);
           } else {
-            mma_f16(me, acc + (nb - 1) * kSkCols, ag, b + (nb - 1) * kDigitStep, idesc(gd), 0u);
-            if (nb > 1) mma_f16(me, acc, ag, b, idesc(nb - 1), 1u);
+            mma_f16_by(me, acc + (nb - 1) * kSkCols, ag, b + (nb - 1) * kDigitStep, idesc(gd), 0u);
+            if (nb > 1) mma_f16_by(me, acc, ag, b, idesc(nb - 1), 1u);
           }
 #pragma unroll
           for (int i = 0; i < kSkGroup; ++i) {
             if (i < gd) {
 #pragma unroll
               for (int kk = i == 0 ? 1 : 0; kk < KS; ++kk)
-                mma_f16(me, acc, ag + i * (kTileBytes >> 4) + 2 * kk, b - i * kDigitStep + 2 * kk, all, 1u);
+                mma_f16_by(me, acc, ag + i * (kTileBytes >> 4) + 2 * kk, b - i * kDigitStep + 2 * kk, all, 1u);
             }
           }
         }

@@ -7,12 +7,12 @@
 // residue path's time is storing and reading back A's digit planes
 // (16384×16×16384, r = 12: 2.03 ms to write 8 GB, 1.36 ms to read them).  Here
 // A is read once per 16 columns and nothing of it is written: a thread
-// quantises 8 entries of a row (Eq. scale), writes their 8 balanced base-256
-// digits as f16 operand tiles to shared memory, and one MMA per digit adds its
-// products with every digit of the skinny operand to the accumulators of their
-// weights.  The sums of 128 k-entries stay exact in FP32 (8 digit pairs · 128 ·
-// 2^14 = 2^24); the accumulators are then added to the integer X_ij that a
-// thread keeps in registers, 160 bits wide, while the tensor core goes on in
+// quantises 8 entries of a row (Eq. scale), writes their balanced base-256
+// digits, up to 8, as f16 operand tiles to shared memory, and one MMA per digit
+// adds its products with every digit of the skinny operand to the accumulators
+// of their weights.  The sums of 128 k-entries stay exact in FP32 (8 digit pairs
+// · 128 · 2^14 = 2^24); the accumulators are then added to the integer X_ij that
+// a thread keeps in registers, 160 bits wide, while the tensor core goes on in
 // the other buffer.  X is the integer the CRT would return, rounded alike: the
 // same bits of C.
 //
@@ -23,11 +23,12 @@
 //
 // With few rows of C instead, B takes A's place (its columns are the rows).
 //
-// Measured on one GB300, 16384×16×16384, r = 12: 0.76 ms for this kernel (2.15
-// GB read once, 0.32 ms at the copy rate) against 2.03 + 1.36 for the planes;
-// the call 4.21 → 1.57 ms (0.71 with seven digits of A instead of eight).  The converting warps' integer pipe bounds it (62
-// instructions per entry, 60% busy, the loads' latency next: a second chunk in
-// flight spills at the 96 registers 18 warps allow and is slower).
+// Measured on one GB300, 16384×16×16384, r = 12 (seven digits of A): 0.72 ms
+// for this kernel (2.15 GB read once, 0.32 ms at the copy rate) against 2.03 +
+// 1.36 for the planes; the call 4.32 → 1.39 ms, the "+1" pass below included.
+// The converting warps' integer pipe bounds it (62 instructions per entry, 60%
+// busy, the loads' latency next: a second chunk in flight spills at the 96
+// registers 18 warps allow and is slower).
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -173,26 +174,6 @@ __global__ void __launch_bounds__(256) skinny_digits_kernel(const double* __rest
 // ---------------------------------------------------------------------------
 // The products.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void sn_mma(uint32_t me, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
-      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(me)
-      : "memory");
-}
-__device__ __forceinline__ void sn_commit(uint32_t me, uint32_t bar) {
-  asm volatile(
-      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
-      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
-      "r"(me)
-      : "memory");
-}
-__device__ __forceinline__ long long sn_mad_wide(int a, int b, long long c) {
-  long long r;
-  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
-  return r;
-}
 __device__ __forceinline__ void mma_f8_by(uint32_t me, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                           uint32_t accumulate) {
   asm volatile(
@@ -346,34 +327,34 @@ __global__ void __launch_bounds__(kSnThreads, 1) skinny_kernel(const __grid_cons
           const uint64_t ag = ab + i0 * (kSnADigit >> 4);
           if (c == 0) {  // the slab's first products: overwrite the weights met for the first time
             if (i0 == 0) {
-              sn_mma(me, acc, ag, bb, all, 0u);
+              mma_f16_by(me, acc, ag, bb, all, 0u);
             } else {
-              sn_mma(me, acc + (nb - 1) * kSnCols, ag, bb + (nb - 1) * kDigitStep, idesc(gd), 0u);
-              if (nb > 1) sn_mma(me, acc, ag, bb, idesc(nb - 1), 1u);
+              mma_f16_by(me, acc + (nb - 1) * kSnCols, ag, bb + (nb - 1) * kDigitStep, idesc(gd), 0u);
+              if (nb > 1) mma_f16_by(me, acc, ag, bb, idesc(nb - 1), 1u);
             }
           } else {
-            sn_mma(me, acc, ag, bb, all, 1u);
+            mma_f16_by(me, acc, ag, bb, all, 1u);
           }
 #pragma unroll
           for (int i = 0; i < kSnGroup; ++i) {
             if (i < gd) {
 #pragma unroll
               for (int kk = i == 0 ? 1 : 0; kk < kSnK / 16; ++kk)
-                sn_mma(me, acc, ag + i * (kSnADigit >> 4) + kk * (2 * kSnATile >> 4),
+                mma_f16_by(me, acc, ag + i * (kSnADigit >> 4) + kk * (2 * kSnATile >> 4),
                        bb - i * kDigitStep + kk * (2 * kSnBTile >> 4), all, 1u);
             }
           }
         }
-        sn_commit(me, aempty + 8 * b);
-        sn_commit(me, bempty + 8 * s);
+        mma_commit_by(me, aempty + 8 * b);
+        mma_commit_by(me, bempty + 8 * s);
       }
-      if (ok) sn_commit(me, accf + 8 * buf);
+      if (ok) mma_commit_by(me, accf + 8 * buf);
     }
     if (!ok && me) {
       a.dev->status = kStatusTimeout;
       a.dev->timeout_site = 15;
     }
-    sn_commit(me, drain_bar);  // every MMA retired before the tensor memory goes away
+    mma_commit_by(me, drain_bar);  // every MMA retired before the tensor memory goes away
     mbar_wait_bounded(drain_bar, 0, kWaitLimit);
     __syncwarp();
   } else {
@@ -415,7 +396,7 @@ __global__ void __launch_bounds__(kSnThreads, 1) skinny_kernel(const __grid_cons
               long long s = static_cast<long long>(carry) + static_cast<long long>(X[j2 + j][g]);
 #pragma unroll
               for (int i = 0; i < 4; ++i)
-                if (4 * g + i < W) s = sn_mad_wide(__float2int_rn(__uint_as_float(v[4 * g + i][j])), a.pow256[i], s);
+                if (4 * g + i < W) s = mad_wide(__float2int_rn(__uint_as_float(v[4 * g + i][j])), a.pow256[i], s);
               X[j2 + j][g] = static_cast<uint32_t>(s);
               carry = static_cast<int>(s >> 32);
             }
@@ -680,10 +661,10 @@ __global__ void __launch_bounds__(kSpThreads, 2) skinny_plus_one_kernel(const __
       for (int kk = 0; kk < kSpK / 32; ++kk)
         mma_f8_by(me, tmem, da + s * (kSpABuf >> 4) + kk * (2 * kSpATile >> 4),
                   db + s * (kSpBBuf >> 4) + kk * (2 * a.npad * 16 >> 4), idesc, kk ? 1u : fresh);
-      sn_commit(me, empty + 8 * s);
+      mma_commit_by(me, empty + 8 * s);
       fresh = 1;
       if (++chunk == a.chunks || t + 1 == units) {
-        sn_commit(me, accf);
+        mma_commit_by(me, accf);
         chunk = 0;
         fresh = 0;
         ++blocks;
@@ -693,7 +674,7 @@ __global__ void __launch_bounds__(kSpThreads, 2) skinny_plus_one_kernel(const __
       a.dev->status = kStatusTimeout;
       a.dev->timeout_site = 18;
     }
-    sn_commit(me, drain_bar);
+    mma_commit_by(me, drain_bar);
     mbar_wait_bounded(drain_bar, 0, kWaitLimit);
     __syncwarp();
   } else {
