@@ -112,7 +112,12 @@ typedef struct {
 /* C = A·B (overwrite, β = 0) by Ozaki Scheme II with TZ quantiser and R2
  * scales.  Allocates its workspace stream-ordered on `stream` from the
  * library's memory pool (see oz2_trim_memory) and frees it on the same
- * stream.  m == 0 or n == 0: no-op; k == 0: C = 0. */
+ * stream.  m == 0 or n == 0: no-op; k == 0: C = 0.  Calls on several streams
+ * may overlap.  This entry and oz2_dgemm_host are the fast ones for k ≤ 64 and
+ * for few rows or columns of C (up to 64 at num_moduli = 12), where they form
+ * the same C without digit planes and residues: 16384²×64 2.2 ms a call against
+ * 4.9 through oz2_dgemm_ex, 16384×16×16384 1.4 against 4.2 (one GB300).  The
+ * entries whose workspace is the caller's or fixed always form both. */
 int oz2_dgemm(int64_t m, int64_t n, int64_t k,
               const double* d_A, int64_t lda,
               const double* d_B, int64_t ldb,
